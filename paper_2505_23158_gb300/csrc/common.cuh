@@ -173,7 +173,7 @@ void launch_chunk_union(const uint32_t* a, int64_t na, const uint32_t* b, int64_
 // K3: projection + SH + visibility compaction.
 struct ProjectOut {
     float4* rec_a;      // (mean'x, mean'y, u00, u01)
-    float4* rec_b;      // (u11, log2 opacity', r, g)
+    float4* rec_b;      // (u11, -log2 opacity', r, g)
     float* rec_c;       // b
     uint2* rec_rect;    // pixel range (x0 | y0 << 16, x1 | y1 << 16), inclusive
     uint32_t* rec_gid;  // gid of the record
@@ -298,8 +298,8 @@ void launch_ranges(const uint32_t* tile_key, int64_t n_keys, uint2* ranges, int6
                    int shift, cudaStream_t s);
 
 // Alpha of a projection record at a pixel (Eq. 1 with the record's
-// Cholesky form): alpha = min(0.99, 2^(log2 o' - (u00 dx + u01 dy)^2 -
-// (u11 dy)^2)), a = (mean', u00, u01), b = (u11, log2 o', ...).  The
+// Cholesky form): alpha = min(0.99, 2^-((u00 dx + u01 dy)^2 + (u11 dy)^2 -
+// log2 o')), a = (mean', u00, u01), b = (u11, -log2 o', ...).  The
 // compositing thread owns the pixels of rows y and y + 4 of an 8-row block
 // and forms the second row's t and w from the first's by the row step (one
 // FMA each), so a pixel whose row within its tile has bit 2 set takes that
@@ -312,7 +312,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 __device__ __forceinline__ float alpha_of(float4 b, float t, float w) {
-    return fminf(0.99f, ex2_approx(fmaf(-t, t, fmaf(-w, w, b.y))));
+    return fminf(0.99f, ex2_approx(-fmaf(t, t, fmaf(w, w, b.y))));
 }
 // t and w at row py0 (a pixel-centre y) and at py0 + 4
 __device__ __forceinline__ void row_pair_tw(float4 a, float4 b, float dx, float py0, float& t0, float& w0,
@@ -346,24 +346,23 @@ struct BlendOut {
 };
 // tile_val[i] & vmask is the record of sorted pair i (vmask = all ones for
 // separate values, the low rbits for packed keys).
-// bin_log2 > 0: ranges and keys are per bin of 2^bin_log2 x 2^bin_log2
-// tiles (launch_emit); a tile walks its bin's list and skips the records
-// whose tile rect (from rec_rect) misses it, which leaves exactly the
+// rec_rect: the records' pixel rects.  bin_log2 > 0: ranges and keys are per
+// bin of 2^bin_log2 x 2^bin_log2 tiles (launch_emit); a tile walks its bin's
+// list and skips the records whose rect misses it, which leaves exactly the
 // tile's own list, in the same order.
 void launch_blend(const DevCamera& cam, const uint2* ranges, const uint32_t* tile_val, uint32_t vmask,
                   int64_t n_keys, const float4* rec_a, const float4* rec_b, const float* rec_c,
-                  int64_t n_rec, const BlendOut& o, cudaStream_t s, int bin_log2 = 0,
-                  const uint2* rec_rect = nullptr, unsigned long long* pairs = nullptr,
+                  int64_t n_rec, const BlendOut& o, cudaStream_t s, int bin_log2,
+                  const uint2* rec_rect, unsigned long long* pairs = nullptr,
                   uint32_t* tile_ctr = nullptr);
 // tile_ctr (a zeroed device word) makes the compositing a grid of
 // kBlendCtasPerSM CTAs per SM that take tiles from the counter, so that
 // other streams' kernels keep room on every SM while it runs (used when
 // frames of other slots run at the same time; a lone frame takes one CTA
-// per tile and the whole GPU).  Measured with 1080p chunk
-// frames on four streams: 2 / 3 / 4 / 6 / 8 / 12 CTAs per SM gave 5790 /
-// 5936 / 5894 / 5775 / 5706 / 5729 frames/s; the single-frame compositing
-// time grows from 0.081 ms at 8 to 0.090 ms at 4).
-constexpr int kBlendCtasPerSM = 4;
+// per tile and the whole GPU).  Eight CTAs fill an SM's registers.  Measured
+// with 3 / 4 / 6 / 8 CTAs per SM: 24 chunk frames at 1080p in 3374 / 3416 /
+// 3408 / 3700 us, four at 4K in 1433 / 1404 / 1359 / 1455 us.
+constexpr int kBlendCtasPerSM = 6;
 // Everything one frame's compositing reads and writes; a batch of frames is
 // composited by one launch over all their tiles (at most kMaxBlendBatch);
 // frames of a batch write images only (no T_final, no last).
@@ -374,7 +373,7 @@ struct BlendFrame {
     int32_t bin_log2, bins_x;  // key lists per bin of 2^bin_log2 tiles square
     const uint2* ranges;       // per bin
     const uint32_t* tile_val;
-    const uint2* rec_rect;     // pixel ranges (read when bin_log2 > 0)
+    const uint2* rec_rect;     // pixel ranges
     unsigned long long* pairs; // null, or [0] += pairs evaluated, [1] += pairs composited
     const float4* rec_a;
     const float4* rec_b;
@@ -390,7 +389,7 @@ struct BlendBatch {
 };
 BlendFrame blend_frame(const DevCamera& cam, const uint2* ranges, const uint32_t* tile_val, uint32_t vmask,
                        int64_t n_keys, const float4* rec_a, const float4* rec_b, const float* rec_c,
-                       int64_t n_rec, const BlendOut& o, int bin_log2 = 0, const uint2* rec_rect = nullptr);
+                       int64_t n_rec, const BlendOut& o, int bin_log2, const uint2* rec_rect);
 // One launch composites every frame's tiles.  With tile_ctr (a zeroed device
 // word) the launch is persistent: a grid of a few CTAs per SM takes (frame,
 // tile) items from the counter until all are done; without it, one CTA per

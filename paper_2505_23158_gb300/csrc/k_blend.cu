@@ -5,29 +5,40 @@
 // pixels terminate together.  The tile's Gaussians arrive in batches of 128
 // records, gathered from the projection records into shared memory with
 // cp.async and double-buffered (batch b+1 is in flight while batch b is
-// composited).  A pixel stops at the first Gaussian that would take its
-// transmittance below 1e-4; a warp whose 64 pixels have all stopped skips
-// the batch, and the CTA leaves as soon as all 256 have stopped.
+// composited; the keys of batch b+2 are already being read, so that no
+// thread waits for a key before it can start a gather).
 //
-// Frames that keep neither the final transmittance nor list positions take
-// the filtered walk: each batch also stages the records' pixel rects, and
-// every warp ballots which of the 128 records have a pixel rect meeting its
-// own 8x8 block and an ellipse reaching one of its pixel centres
-// (splat_meets_block), and visits only those, in list order.  A record
-// failing either test would be skipped by every pixel of the block (alpha <
-// 1/255 there), so the image is the unfiltered walk's bit for bit.
-// With coarse bins (squares of 2^bin_log2 tiles) the tile walks its bin's
-// key list the same way (a record meeting the block has a tile rect holding
-// the tile, so it is on the tile's own list).  This walk is branch-free: a
-// pixel that stops gets T = 0, which makes every later step a no-op.
+// Filtered walk: each thread tests the record it staged against the tile's
+// four 8x8 blocks (walk.cuh, blocks_met), the warps ballot the results, and
+// every warp makes a list of the records that can reach its own block and
+// visits only those, in list order.  A record failing the test would be
+// skipped by every pixel of the block (alpha < 1/255 there), so the image is
+// that of walking the whole list, bit for bit.  With coarse bins (squares of
+// 2^bin_log2 tiles) the tile walks its bin's key list the same way (a record
+// meeting a block has a tile rect holding the tile, so it is on the tile's
+// own list).
 //
 // Per pixel and Gaussian (record = mean', upper-triangular U with
-// U^T U = (1/2) log2(e) Sigma'^-1, log2 o', colour):
-//   q = (u00 dx + u01 dy)^2 + (u11 dy)^2,  alpha = min(0.99, 2^(log2 o' - q))
-//   (= o' 2^-q; the exponent is formed by two FMAs and the product is saved)
+// U^T U = (1/2) log2(e) Sigma'^-1, -log2 o', colour):
+//   q = (u00 dx + u01 dy)^2 + (u11 dy)^2,  alpha = min(0.99, 2^-(q - log2 o'))
 //   skip if alpha < 1/255; T' = T (1 - alpha); stop if T' < 1e-4;
 //   C += T alpha rgb; T = T'.
-#include "common.cuh"
+// The step has no branches: alpha becomes 0 where the pixel skips (T' = T,
+// weight 0) and T becomes 0 where it stops, which makes every later step a
+// no-op.  A thread's two pixels run in packed FP32 pairs.
+//
+// What bounds it: instruction issue and the FP32 pipes.  A visit of a record
+// by a warp (64 pixels) takes about 38 instructions, 30 FP32 pipe cycles of
+// them, against 58 with scalar steps, the hits taken bit by bit from the
+// masks and every block testing every record for itself.  A 1080p chunk
+// frame of 120k visible records (83M evaluated pairs): 97.1M -> 70.6M warp
+// instructions, 135 -> 102 us (whole GPU to itself); a full-detail frame of
+// 858k records 455 -> 254 us, its longest lists being walked four records at
+// a time instead of one after the other.  Storing the scalars that enter
+// packed steps twice in shared memory measured no fewer FP32 instructions (a
+// packed operand may be one register used twice).  64 registers (8 CTAs per
+// SM): 10 CTAs with 48 measured 2-4% slower, no limit (66-72 registers) 1-3%.
+#include "walk.cuh"
 
 namespace lodge {
 
@@ -36,111 +47,57 @@ namespace {
 constexpr int kBatch = 256;        // importance kernel: records per batch
 constexpr int kBlendThreads = 128; // blend: two pixels per thread
 constexpr int kBlendBatch = 128;   // blend: records per batch (one per thread)
+constexpr int kUnroll = 4;         // records visited per turn of the walk
+constexpr uint32_t kNoHit = 16u * kBlendBatch;   // offset of a record no pixel composites
 
+// two pixels of one thread
+struct PixelPair {
+    f32x2 T, C0, C1, C2;
+};
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
-    unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-    unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::); }
-
-// one record of the batch against one pixel (Eq. 1); kCount: count the
-// evaluation and, if the pixel composites it, the composited pair
-template <bool kCount, bool kLast>
-__device__ __forceinline__ void blend_px(const float alpha, const float4 bb, const float cz, float& T,
-                                         float& C0, float& C1, float& C2, bool& done, uint32_t& last,
-                                         uint32_t pos, uint32_t& n_eval, uint32_t& n_used) {
-    if (kCount) ++n_eval;
-    if (alpha >= (1.0f / 255.0f)) {
-        const float Tn = T * (1.f - alpha);
-        if (Tn < 1e-4f) {
-            done = true;
-        } else {
-            const float wgt = T * alpha;
-            C0 = fmaf(wgt, bb.z, C0);
-            C1 = fmaf(wgt, bb.w, C1);
-            C2 = fmaf(wgt, cz, C2);
-            T = Tn;
-            if (kLast) last = pos;
-            if (kCount) ++n_used;
-        }
-    }
+// One record against the thread's two pixels (Eq. 1).  Returns the weights
+// T alpha (0 where the pixel skips or has stopped) and the transmittances
+// after the record (0 where it has stopped).
+__device__ __forceinline__ void blend_pair(const char* __restrict__ rec, float pxf, float py0, PixelPair& p,
+                                           f32x2& wgt) {
+    constexpr int kNext = sizeof(float4) * (kBlendBatch + 1);
+    const float4 a = *reinterpret_cast<const float4*>(rec);
+    const float4 b = *reinterpret_cast<const float4*>(rec + kNext);
+    const float cz = *reinterpret_cast<const float*>(rec + 2 * kNext);
+    float t0, w0, t1, w1;
+    row_pair_tw(a, b, pxf - a.x, py0, t0, w0, t1, w1);
+    const f32x2 t = pack2(t0, t1), w = pack2(w0, w1);
+    float z0, z1;
+    unpack2(fma2(t, t, fma2(w, w, pack2(b.y, b.y))), z0, z1);
+    const float a0 = fminf(0.99f, ex2_approx(-z0)), a1 = fminf(0.99f, ex2_approx(-z1));
+    // alpha, or 0 below 1/255
+    const f32x2 al = mul2(pack2(a0, a1), pack2(ge01(a0, 1.0f / 255.0f), ge01(a1, 1.0f / 255.0f)));
+    const f32x2 Tn = mul2(p.T, fma2(al, pack2(-1.f, -1.f), pack2(1.f, 1.f)));
+    float n0, n1;
+    unpack2(Tn, n0, n1);
+    const f32x2 go = pack2(ge01(n0, 1e-4f), ge01(n1, 1e-4f));
+    wgt = mul2(mul2(p.T, al), go);
+    p.T = mul2(Tn, go);
+    p.C0 = fma2(wgt, pack2(b.z, b.z), p.C0);
+    p.C1 = fma2(wgt, pack2(b.w, b.w), p.C1);
+    p.C2 = fma2(wgt, pack2(cz, cz), p.C2);
 }
 
-// The same step without branches, for walks that need neither the final
-// transmittance nor list positions: a pixel that stops gets T = 0, after
-// which every step leaves it unchanged (its weight is 0 and T stays 0).
-// While T > 0 the arithmetic and decisions are blend_px's.
-template <bool kCount>
-__device__ __forceinline__ void blend_px_flat(const float alpha, const float4 bb, const float cz, float& T,
-                                              float& C0, float& C1, float& C2, uint32_t& n_eval,
-                                              uint32_t& n_used) {
-    const float Tn = T * (1.f - alpha);
-    const bool ok = alpha >= (1.0f / 255.0f);
-    const bool go = ok && !(Tn < 1e-4f);
-    const float wgt = go ? T * alpha : 0.f;
-    C0 = fmaf(wgt, bb.z, C0);
-    C1 = fmaf(wgt, bb.w, C1);
-    C2 = fmaf(wgt, cz, C2);
-    if (kCount) {
-        n_eval += T > 0.f ? 1u : 0u;
-        n_used += go ? 1u : 0u;
-    }
-    T = go ? Tn : (ok ? 0.f : T);
-}
-
-// Whether a splat can reach alpha >= 1/255 at some pixel centre of an 8x8
-// block whose first pixel centre is (bx, by).  With d = p - mean' and
-// q(d) = (u00 dx + u01 dy)^2 + (u11 dy)^2 (the exponent's quadratic, a convex
-// function with its minimum 0 at d = 0), the least q over the centres' box
-// [bx, bx + 7] x [by, by + 7] lies on the line dx = xc or on dy = yc, where
-// xc, yc are the box coordinates nearest the mean (0 where the box spans it):
-// along each line q is a one-dimensional quadratic whose minimiser is
-// clamped to the box.  A pixel centre can pass the 1/255 skip only if
-// q <= log2 o' + log2 255; the test adds a margin of 0.01 (in log2 units)
-// for the rounding of q, so it never drops a record that some pixel of the
-// block would composite, and the walk's result is the unfiltered walk's.
-__device__ __forceinline__ bool splat_meets_block(const float4 a, const float4 b, float bx, float by) {
-    constexpr float kLog2_255 = 7.99435343f;
-    const float X0 = bx - a.x, X1 = X0 + 7.f, Y0 = by - a.y, Y1 = Y0 + 7.f;
-    const float xc = fminf(fmaxf(0.f, X0), X1), yc = fminf(fmaxf(0.f, Y0), Y1);
-    const float u00 = a.z, u01 = a.w, u11 = b.x;
-    // on dx = xc the minimiser is dy = -u00 u01 xc / (u01^2 + u11^2)
-    const float dy = fminf(fmaxf(__fdividef(-u00 * u01 * xc, fmaf(u01, u01, u11 * u11)), Y0), Y1);
-    const float t1 = fmaf(u00, xc, u01 * dy), w1 = u11 * dy;
-    // on dy = yc it is dx = -u01 yc / u00
-    const float dx = fminf(fmaxf(__fdividef(-u01 * yc, u00), X0), X1);
-    const float t2 = fmaf(u00, dx, u01 * yc), w2 = u11 * yc;
-    const float q = fminf(fmaf(t1, t1, w1 * w1), fmaf(t2, t2, w2 * w2));
-    return q <= b.y + (kLog2_255 + 0.01f);
-}
-
-template <bool kBins, bool kCount = false>
+// kSave: frames kept for the adjoint also store the final transmittance and
+// the list position (1-based) of the last composited record.  kCount: count
+// the evaluated and composited (pixel, Gaussian) pairs.
+template <bool kSave, bool kCount = false>
 __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
-    __shared__ float4 sa[2][kBlendBatch];
-    __shared__ float4 sb[2][kBlendBatch];
-    __shared__ float sc[2][kBlendBatch];
-    __shared__ uint2 sr[2][kBins ? kBlendBatch : 1];
+    __shared__ float4 s_rec[2][3][kBlendBatch + 1];        // the last one composites nowhere
+    __shared__ uint32_t s_met[4][kBlendBatch / 32];        // per block: which records reach it
+    __shared__ __align__(8) uint16_t s_hit[4][kBlendBatch + kUnroll];   // per warp: their offsets
     const int32_t width = f.width, height = f.height, tiles_x = f.tiles_x;
-    const uint2* __restrict__ ranges = f.ranges;
     const uint32_t* __restrict__ tile_val = f.tile_val;
     const uint32_t vmask = f.vmask, n_keys = f.n_keys, n_rec = f.n_rec;
     const float4* __restrict__ rec_a = f.rec_a;
     const float4* __restrict__ rec_b = f.rec_b;
     const float* __restrict__ rec_c = f.rec_c;
-    float* __restrict__ out_rgb = f.rgb;
-    float* __restrict__ out_T = f.T_final;
-    uint32_t* __restrict__ out_last = f.last;
+    const uint2* __restrict__ rec_rect = f.rec_rect;
     const int tx = tile % tiles_x, ty = tile / tiles_x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // warp w covers the 8x8 block (w & 1, w >> 1) of the tile; a lane owns
@@ -149,125 +106,100 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
     const int y0 = ty * kTile + (warp >> 1) * 8 + (lane >> 3), y1 = y0 + 4;
     const bool in0 = x < width && y0 < height, in1 = x < width && y1 < height;
     const float pxf = (float)x + 0.5f, py0 = (float)y0 + 0.5f;
-    const uint32_t wx0 = tx * kTile + (warp & 1) * 8, wx1 = wx0 + 7;   // the warp's 8x8 block
-    const uint32_t wy0 = ty * kTile + (warp >> 1) * 8, wy1 = wy0 + 7;
-    const float bxf = (float)wx0 + 0.5f, byf = (float)wy0 + 0.5f;   // the block's first pixel centre
-    const uint2* __restrict__ rec_rect = f.rec_rect;
-    // the rect test needs the records' pixel rects (frames that keep the
-    // final transmittance or positions have none); a frame of a filtered
-    // batch launch may still have per-tile lists without rects
-    const bool binned = kBins && rec_rect != nullptr;
-    const int bin = (binned && f.bin_log2 > 0) ? (ty >> f.bin_log2) * f.bins_x + (tx >> f.bin_log2) : tile;
-    uint2 rg = ranges[bin];
+    const int bin = f.bin_log2 > 0 ? (ty >> f.bin_log2) * f.bins_x + (tx >> f.bin_log2) : tile;
+    uint2 rg = f.ranges[bin];
     if (rg.y > n_keys || rg.x > rg.y) rg = make_uint2(0, 0);  // never for a consistent sort
     const int n = (int)(rg.y - rg.x);
     const int nb = (n + kBlendBatch - 1) / kBlendBatch;
+    tile_val += rg.x;
 
-    // the binned walk marks a pixel outside the image or stopped by T = 0
-    float T0 = (kBins && !in0) ? 0.f : 1.f, C00 = 0.f, C01 = 0.f, C02 = 0.f;
-    float T1 = (kBins && !in1) ? 0.f : 1.f, C10 = 0.f, C11 = 0.f, C12 = 0.f;
-    bool done0 = !in0, done1 = !in1;
+    // a pixel outside the image counts as stopped (T = 0)
+    PixelPair p{pack2(in0 ? 1.f : 0.f, in1 ? 1.f : 0.f), 0ull, 0ull, 0ull};
+    float Tk0 = 1.f, Tk1 = 1.f;        // kSave: the transmittance behind the last composited record
     uint32_t last0 = 0, last1 = 0;
     uint32_t n_eval = 0, n_used = 0;   // counting mode only
-    // per-pixel list positions are wanted only by the adjoint, whose frames
-    // always have per-tile lists
-    constexpr bool kLast = !kBins;
 
-    if (nb > 0) {
-        if (tid < n) {
-            uint32_t j = min(tile_val[rg.x + tid] & vmask, n_rec - 1u);
-            cp_async16(&sa[0][tid], rec_a + j);
-            cp_async16(&sb[0][tid], rec_b + j);
-            cp_async4(&sc[0][tid], rec_c + j);
-            if (binned) cp_async8(&sr[0][tid], rec_rect + j);
-        }
-        cp_async_commit();
+    auto stopped = [&]() {
+        float T0, T1;
+        unpack2(p.T, T0, T1);
+        return T0 == 0.f && T1 == 0.f;
+    };
+    auto stage = [&](int buf, uint32_t key) {
+        const uint32_t j = min(key & vmask, n_rec - 1u);
+        cp_async16(&s_rec[buf][0][tid], rec_a + j);
+        cp_async16(&s_rec[buf][1][tid], rec_b + j);
+        cp_async4(&s_rec[buf][2][tid].x, rec_c + j);
+        cp_async8(&s_rec[buf][2][tid].z, rec_rect + j);
+    };
+    if (tid < 2) {   // alpha = 2^-inf = 0
+        s_rec[tid][0][kBlendBatch] = make_float4(0.f, 0.f, 0.f, 0.f);
+        s_rec[tid][1][kBlendBatch] = make_float4(0.f, __int_as_float(0x7f800000), 0.f, 0.f);
+        s_rec[tid][2][kBlendBatch] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+    if (tid < n) stage(0, tile_val[tid]);
+    cp_async_commit();
+    uint32_t key = kBlendBatch + tid < n ? tile_val[kBlendBatch + tid] : 0u;
     for (int b = 0; b < nb; ++b) {
         const int buf = b & 1;
-        if (b + 1 < nb) {
-            int k = (b + 1) * kBlendBatch + tid;
-            if (k < n) {
-                uint32_t j = min(tile_val[rg.x + k] & vmask, n_rec - 1u);
-                cp_async16(&sa[buf ^ 1][tid], rec_a + j);
-                cp_async16(&sb[buf ^ 1][tid], rec_b + j);
-                cp_async4(&sc[buf ^ 1][tid], rec_c + j);
-                if (binned) cp_async8(&sr[buf ^ 1][tid], rec_rect + j);
-            }
-        }
+        const int k1 = (b + 1) * kBlendBatch + tid;
+        if (k1 < n) stage(buf ^ 1, key);
         cp_async_commit();
+        key = k1 + kBlendBatch < n ? tile_val[k1 + kBlendBatch] : 0u;
         cp_async_wait1();
+        {   // the record this thread staged against the tile's four blocks
+            uint32_t met = 0;
+            if (b * kBlendBatch + tid < n) {
+                const float4 c = s_rec[buf][2][tid];
+                met = blocks_met(s_rec[buf][0][tid], s_rec[buf][1][tid],
+                                 make_uint2(__float_as_uint(c.z), __float_as_uint(c.w)), tx * kTile, ty * kTile);
+            }
+            uint32_t m = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t v = __ballot_sync(0xffffffffu, met >> q & 1u);
+                if (lane == q) m = v;
+            }
+            if (lane < 4) s_met[lane][warp] = m;
+        }
         __syncthreads();
-        const int cnt = min(kBlendBatch, n - b * kBlendBatch);
-        if (kBins) {
-            // which records of the batch can reach this warp's block: 4
-            // ballots per warp
-            uint32_t m[kBlendBatch / 32];
+        if (!__all_sync(0xffffffffu, stopped())) {
+            // the records that can reach this warp's block, in list order
+            int nh = 0;
 #pragma unroll
             for (int w = 0; w < kBlendBatch / 32; ++w) {
-                const int k = w * 32 + lane;
-                bool hit = k < cnt;
-                if (hit && binned) {
-                    // the record's pixel rect meets this warp's 8x8 block (so
-                    // its tile rect holds the tile); outside the rect every
-                    // pixel would skip it (alpha < 1/255), so no result changes
-                    const uint2 r = sr[buf][k];
-                    hit = (r.x & 0xffffu) <= wx1 && (r.y & 0xffffu) >= wx0 && (r.x >> 16) <= wy1 &&
-                          (r.y >> 16) >= wy0;
-                }
-                // and its ellipse reaches a pixel centre of the block
-                if (hit) hit = splat_meets_block(sa[buf][k], sb[buf][k], bxf, byf);
-                m[w] = __ballot_sync(0xffffffffu, hit);
+                const uint32_t m = s_met[warp][w];
+                if (m >> lane & 1u)
+                    s_hit[warp][nh + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(16 * (w * 32 + lane));
+                nh += __popc(m);
             }
-            // flat walk over the hits, 8 batch positions at a time, the warp
-            // leaving once all its pixels have stopped (T = 0)
-            if (!__all_sync(0xffffffffu, T0 == 0.f && T1 == 0.f)) {
-                // the hits in batch order, taken bit by bit from the masks
-                // (a warp visits a quarter or less of a staged batch; a scan
-                // over all 128 positions with a test each cost more)
-                bool open = true;
+            if (lane < kUnroll) s_hit[warp][nh + lane] = (uint16_t)kNoHit;
+            __syncwarp();
+            const char* base = reinterpret_cast<const char*>(&s_rec[buf][0][0]);
+            for (int i = 0; i < nh; i += kUnroll) {
+                const uint2 h = *reinterpret_cast<const uint2*>(&s_hit[warp][i]);
+                const uint32_t off[kUnroll] = {h.x & 0xffffu, h.x >> 16, h.y & 0xffffu, h.y >> 16};
 #pragma unroll
-                for (int w = 0; w < kBlendBatch / 32; ++w) {
-                    uint32_t mw = open ? m[w] : 0u;
-                    uint32_t cnt8 = 0;
-                    while (mw) {
-                        const int k = w * 32 + __ffs(mw) - 1;
-                        mw &= mw - 1u;
-                        const float4 a = sa[buf][k];
-                        const float4 bb = sb[buf][k];
-                        const float cz = sc[buf][k];
-                        float t0, w0, t1, w1;
-                        row_pair_tw(a, bb, pxf - a.x, py0, t0, w0, t1, w1);
-                        blend_px_flat<kCount>(alpha_of(bb, t0, w0), bb, cz, T0, C00, C01, C02, n_eval, n_used);
-                        blend_px_flat<kCount>(alpha_of(bb, t1, w1), bb, cz, T1, C10, C11, C12, n_eval, n_used);
-                        if ((++cnt8 & 7u) == 0u && __all_sync(0xffffffffu, T0 == 0.f && T1 == 0.f)) {
-                            open = false;
-                            break;
-                        }
+                for (int u = 0; u < kUnroll; ++u) {
+                    f32x2 wgt;
+                    if (kCount && off[u] != kNoHit) {
+                        float T0, T1;
+                        unpack2(p.T, T0, T1);
+                        n_eval += (T0 > 0.f ? 1u : 0u) + (T1 > 0.f ? 1u : 0u);
+                    }
+                    blend_pair(base + off[u], pxf, py0, p, wgt);
+                    if (kSave || kCount) {
+                        float w0, w1, T0, T1;
+                        unpack2(wgt, w0, w1);
+                        unpack2(p.T, T0, T1);
+                        const uint32_t pos = (uint32_t)(b * kBlendBatch + 1) + off[u] / 16u;
+                        if (w0 > 0.f) { Tk0 = T0; last0 = pos; ++n_used; }
+                        if (w1 > 0.f) { Tk1 = T1; last1 = pos; ++n_used; }
                     }
                 }
-            }
-        } else if (!__all_sync(0xffffffffu, done0 && done1)) {
-            for (int k = 0; k < cnt && !(done0 && done1); ++k) {
-                const float4 a = sa[buf][k];
-                const float4 bb = sb[buf][k];
-                const float cz = sc[buf][k];
-                const uint32_t pos = (uint32_t)(b * kBlendBatch + k + 1);
-                float t0, w0, t1, w1;
-                row_pair_tw(a, bb, pxf - a.x, py0, t0, w0, t1, w1);
-                if (!done0)
-                    blend_px<kCount, kLast>(alpha_of(bb, t0, w0), bb, cz, T0, C00, C01, C02, done0, last0, pos,
-                                            n_eval, n_used);
-                if (!done1)
-                    blend_px<kCount, kLast>(alpha_of(bb, t1, w1), bb, cz, T1, C10, C11, C12, done1, last1, pos,
-                                            n_eval, n_used);
+                if (__all_sync(0xffffffffu, stopped())) break;
             }
         }
-        if (kBins) {
-            if (__syncthreads_count(T0 == 0.f && T1 == 0.f) == kBlendThreads) break;
-        } else if (__syncthreads_count(done0 && done1) == kBlendThreads) {
-            break;
-        }
+        if (__syncthreads_count(stopped()) == kBlendThreads) break;
     }
     cp_async_wait0();
     if (kCount) {
@@ -280,32 +212,34 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
             atomicAdd(f.pairs + 1, (unsigned long long)n_used);
         }
     }
+    float r0, r1, g0, g1, b0, b1;
+    unpack2(p.C0, r0, r1);
+    unpack2(p.C1, g0, g1);
+    unpack2(p.C2, b0, b1);
     if (in0) {
         const int64_t pix = (int64_t)y0 * width + x;
-        out_rgb[3 * pix + 0] = C00;
-        out_rgb[3 * pix + 1] = C01;
-        out_rgb[3 * pix + 2] = C02;
-        if (!kBins && out_T) out_T[pix] = T0;
-        if (kLast && out_last) out_last[pix] = last0;
+        f.rgb[3 * pix + 0] = r0;
+        f.rgb[3 * pix + 1] = g0;
+        f.rgb[3 * pix + 2] = b0;
+        if (kSave) { f.T_final[pix] = Tk0; f.last[pix] = last0; }
     }
     if (in1) {
         const int64_t pix = (int64_t)y1 * width + x;
-        out_rgb[3 * pix + 0] = C10;
-        out_rgb[3 * pix + 1] = C11;
-        out_rgb[3 * pix + 2] = C12;
-        if (!kBins && out_T) out_T[pix] = T1;
-        if (kLast && out_last) out_last[pix] = last1;
+        f.rgb[3 * pix + 0] = r1;
+        f.rgb[3 * pix + 1] = g1;
+        f.rgb[3 * pix + 2] = b1;
+        if (kSave) { f.T_final[pix] = Tk1; f.last[pix] = last1; }
     }
 }
 
-template <bool kBins, bool kCount>
-__global__ void __launch_bounds__(kBlendThreads) blend_kernel(BlendFrame f) {
-    blend_tile<kBins, kCount>(f, blockIdx.x);
+template <bool kSave, bool kCount>
+__global__ void __launch_bounds__(kBlendThreads, 8) blend_kernel(BlendFrame f) {
+    blend_tile<kSave, kCount>(f, blockIdx.x);
 }
 
 // fewer CTAs than tiles: each takes the next tile from the counter
-template <bool kBins, bool kCount>
-__global__ void __launch_bounds__(kBlendThreads) blend_loop_kernel(BlendFrame f, uint32_t* __restrict__ tile_ctr) {
+template <bool kCount>
+__global__ void __launch_bounds__(kBlendThreads, 8) blend_loop_kernel(BlendFrame f, uint32_t* __restrict__ tile_ctr) {
     __shared__ int s_t;
     for (;;) {
         if (threadIdx.x == 0) s_t = (int)atomicAdd(tile_ctr, 1u);
@@ -313,27 +247,25 @@ __global__ void __launch_bounds__(kBlendThreads) blend_loop_kernel(BlendFrame f,
         const int t = s_t;
         __syncthreads();   // s_t is rewritten for the next tile
         if (t >= f.ntiles) break;
-        blend_tile<kBins, kCount>(f, t);
+        blend_tile<false, kCount>(f, t);
     }
 }
 
 // One launch for the tiles of several frames (a serving step): CTA b
 // composites tile b - tile_base of the last frame whose tile_base <= b.
-template <bool kBins>
-__global__ void __launch_bounds__(kBlendThreads) blend_batch_kernel(BlendBatch bb) {
+__global__ void __launch_bounds__(kBlendThreads, 8) blend_batch_kernel(BlendBatch bb) {
     const uint32_t b = blockIdx.x;
     int lo = 0, hi = bb.n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (bb.f[mid].tile_base <= b) lo = mid; else hi = mid - 1;
     }
-    blend_tile<kBins>(bb.f[lo], (int)(b - bb.f[lo].tile_base));
+    blend_tile<false>(bb.f[lo], (int)(b - bb.f[lo].tile_base));
 }
 
 // The same as a persistent grid: each CTA takes the next (frame, tile) item
 // of the step from the counter until all `total` are done.
-template <bool kBins>
-__global__ void __launch_bounds__(kBlendThreads) blend_batch_loop_kernel(BlendBatch bb, uint32_t total,
+__global__ void __launch_bounds__(kBlendThreads, 8) blend_batch_loop_kernel(BlendBatch bb, uint32_t total,
                                                                          uint32_t* __restrict__ tile_ctr) {
     __shared__ uint32_t s_t;
     for (;;) {
@@ -347,7 +279,7 @@ __global__ void __launch_bounds__(kBlendThreads) blend_batch_loop_kernel(BlendBa
             const int mid = (lo + hi + 1) >> 1;
             if (bb.f[mid].tile_base <= b) lo = mid; else hi = mid - 1;
         }
-        blend_tile<kBins>(bb.f[lo], (int)(b - bb.f[lo].tile_base));
+        blend_tile<false>(bb.f[lo], (int)(b - bb.f[lo].tile_base));
     }
 }
 
@@ -454,13 +386,11 @@ BlendFrame blend_frame(const DevCamera& cam, const uint2* ranges, const uint32_t
     f.vmask = vmask;
     f.n_keys = (uint32_t)n_keys;
     f.n_rec = (uint32_t)std::max<int64_t>(n_rec, 1);
-    // the filtered walk keeps neither the final transmittance nor positions
-    const bool filt = rec_rect && !o.T_final && !o.last;
-    f.bin_log2 = filt ? bin_log2 : 0;
+    f.bin_log2 = bin_log2;
     f.bins_x = (cam.tiles_x + (1 << f.bin_log2) - 1) >> f.bin_log2;
     f.ranges = ranges;
     f.tile_val = tile_val;
-    f.rec_rect = filt ? rec_rect : nullptr;
+    f.rec_rect = rec_rect;
     f.pairs = nullptr;
     f.rec_a = rec_a;
     f.rec_b = rec_b;
@@ -483,25 +413,19 @@ void launch_blend(const DevCamera& cam, const uint2* ranges, const uint32_t* til
     if (tile_ctr) {
         grid = (unsigned)std::min<int64_t>(f.ntiles, (int64_t)device_sms() * kBlendCtasPerSM);
     }
-    const bool filt = f.rec_rect != nullptr;
-    if (tile_ctr) {
-        if (pairs) {   // counting variant (profiling), same walk
-            if (filt)
-                blend_loop_kernel<true, true><<<grid, kBlendThreads, 0, s>>>(f, tile_ctr);
-            else
-                blend_loop_kernel<false, true><<<grid, kBlendThreads, 0, s>>>(f, tile_ctr);
-        } else if (filt) {
-            blend_loop_kernel<true, false><<<grid, kBlendThreads, 0, s>>>(f, tile_ctr);
-        } else {
-            blend_loop_kernel<false, false><<<grid, kBlendThreads, 0, s>>>(f, tile_ctr);
-        }
-    } else if (pairs) {
-        if (filt)
-            blend_kernel<true, true><<<grid, kBlendThreads, 0, s>>>(f);
+    const bool save = o.T_final != nullptr;   // (always a lone frame)
+    if (save) {
+        if (pairs)
+            blend_kernel<true, true><<<(unsigned)f.ntiles, kBlendThreads, 0, s>>>(f);
         else
-            blend_kernel<false, true><<<grid, kBlendThreads, 0, s>>>(f);
-    } else if (filt) {
-        blend_kernel<true, false><<<grid, kBlendThreads, 0, s>>>(f);
+            blend_kernel<true, false><<<(unsigned)f.ntiles, kBlendThreads, 0, s>>>(f);
+    } else if (tile_ctr) {
+        if (pairs)   // counting variant (profiling), same walk
+            blend_loop_kernel<true><<<grid, kBlendThreads, 0, s>>>(f, tile_ctr);
+        else
+            blend_loop_kernel<false><<<grid, kBlendThreads, 0, s>>>(f, tile_ctr);
+    } else if (pairs) {
+        blend_kernel<false, true><<<grid, kBlendThreads, 0, s>>>(f);
     } else {
         blend_kernel<false, false><<<grid, kBlendThreads, 0, s>>>(f);
     }
@@ -511,13 +435,11 @@ void launch_blend_batch(const BlendFrame* frames, int n, cudaStream_t s, uint32_
     BlendBatch bb;
     uint32_t base = 0;
     bb.n = 0;
-    bool bins = false;   // the filtered walk also serves frames without rects
     for (int i = 0; i < n && i < kMaxBlendBatch; ++i) {
         if (frames[i].ntiles == 0) continue;
         bb.f[bb.n] = frames[i];
         bb.f[bb.n].tile_base = base;
         base += (uint32_t)frames[i].ntiles;
-        bins = bins || frames[i].rec_rect != nullptr;
         ++bb.n;
     }
     if (bb.n == 0) return;
@@ -526,21 +448,12 @@ void launch_blend_batch(const BlendFrame* frames, int n, cudaStream_t s, uint32_
         // runs after every frame's earlier stages)
         int per_sm = 1;
         const int nsm = device_sms();
-        if (bins)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, blend_batch_loop_kernel<true>, kBlendThreads, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, blend_batch_loop_kernel<false>, kBlendThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, blend_batch_loop_kernel, kBlendThreads, 0);
         const unsigned grid = (unsigned)std::min<int64_t>((int64_t)base, (int64_t)nsm * std::max(per_sm, 1));
-        if (bins)
-            blend_batch_loop_kernel<true><<<grid, kBlendThreads, 0, s>>>(bb, base, tile_ctr);
-        else
-            blend_batch_loop_kernel<false><<<grid, kBlendThreads, 0, s>>>(bb, base, tile_ctr);
+        blend_batch_loop_kernel<<<grid, kBlendThreads, 0, s>>>(bb, base, tile_ctr);
         return;
     }
-    if (bins)
-        blend_batch_kernel<true><<<base, kBlendThreads, 0, s>>>(bb);
-    else
-        blend_batch_kernel<false><<<base, kBlendThreads, 0, s>>>(bb);
+    blend_batch_kernel<<<base, kBlendThreads, 0, s>>>(bb);
 }
 
 void launch_importance(const DevCamera& cam, const uint2* ranges, const uint32_t* tile_val,

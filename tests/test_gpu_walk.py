@@ -1,0 +1,64 @@
+"""The walks over a tile's key list at the sizes where they can go wrong:
+list lengths around a staged batch (128 records) and a turn of the walk (4),
+on images that are not whole blocks or tiles, against the FP64 oracle.
+
+Bars: pixels max-abs 2e-4 and mean-abs 1e-5 with knife-edge pixels checked
+against the oracle's reachable range, as in the parity tests."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2505_23158_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2505_23158_gb300 import build
+    build.build()
+    from paper_2505_23158_gb300 import api
+    ctx = api.Lodge(0)
+    yield torch, api, ctx
+    ctx.close()
+
+
+def _stack_scene(n, seed, opacity=-3.0):
+    """n faint, anisotropic Gaussians on the view axis: every pixel of a
+    small image composites most of them without saturating."""
+    r = np.random.default_rng(seed)
+    means = np.zeros((n, 3), np.float32)
+    means[:, :2] = r.normal(0, 0.25, (n, 2))
+    means[:, 2] = r.uniform(-1, 1, n)
+    lv = synth.Level(means, r.normal(-2.2, 0.7, (n, 3)).astype(np.float32),
+                     r.normal(size=(n, 4)).astype(np.float32),
+                     r.normal(opacity, 0.5, n).astype(np.float32),
+                     r.normal(0, 0.3, (n, 16, 3)).astype(np.float32))
+    return synth.Scene(levels=[lv], d_thresholds=np.zeros(0), chunk_centers=np.zeros((1, 3)))
+
+
+@pytest.mark.parametrize("n,wh", [(1, (8, 8)), (3, (16, 16)), (4, (7, 9)), (5, (31, 17)), (127, (16, 16)),
+                                  (128, (15, 16)), (129, (33, 16)), (131, (16, 40)), (256, (24, 24)),
+                                  (257, (9, 23)), (1000, (40, 33))])
+def test_list_lengths(env, n, wh):
+    torch, api, ctx = env
+    scene = _stack_scene(n, n)
+    cam = synth.look_at((0.0, 0.0, -3.0), (0.0, 0.0, 1.0), (0.0, -1.0, 0.0), wh[0], wh[1], 30.0)
+    osc = O.OracleScene(scene)
+    ref = O.render(osc, cam, np.arange(n))
+    sid = ctx.load_scene(scene)
+    try:
+        for log2 in (0, 1, 3):
+            ctx.set_bin_size(log2)
+            img, st = ctx.render(sid, api.FULL, cam)
+            assert st["n_visible"] == ref["n_visible"] and st["n_keys"] == ref["n_keys"]
+            O.compare_pixels(img.cpu().numpy(), ref, max_abs=2e-4, mean_abs=1e-5)
+            saved, _, h = ctx.render(sid, api.FULL, cam, save=True)
+            ctx.release(h)
+            assert torch.equal(img, saved)
+    finally:
+        ctx.set_bin_size(-1)
+        ctx.unload_scene(sid)
