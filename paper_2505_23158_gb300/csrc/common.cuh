@@ -406,10 +406,10 @@ void launch_importance(const DevCamera& cam, const uint2* ranges, const uint32_t
                        uint32_t* rec_score, int64_t n_total, float* score, cudaStream_t s);
 
 // K8 / K9: adjoint of compositing and projection (fine-tuning path).
-// grec: 9 x n_rec doubles, zeroed: d(mean'x, mean'y, u00, u01, u11, o', r, g, b).
+// grec: n_rec x 9 doubles, zeroed: the adjoint sums of each record (k_backward.cu).
 void launch_blend_bwd(const DevCamera& cam, const uint2* ranges, const uint32_t* tile_val,
                       uint32_t vmask, int64_t n_keys, const float4* rec_a, const float4* rec_b, const float* rec_c,
-                      int64_t n_rec, const float* T_final, const uint32_t* last,
+                      int64_t n_rec, const uint2* rec_rect, const float* T_final, const uint32_t* last,
                       const float* dL_drgb, double* grec, cudaStream_t s);
 // Levels of a parameter frame as the adjoint sees them: the Eq. 3 filter
 // variance of each level (gid ranges level_off) and the trained level's gid

@@ -55,6 +55,14 @@ struct PixelPair {
     f32x2 T, C0, C1, C2;
 };
 
+// per half: a where the flag is set, else b
+__device__ __forceinline__ f32x2 keep2(bool lo, bool hi, f32x2 a, f32x2 b) {
+    float a0, a1, b0, b1;
+    unpack2(a, a0, a1);
+    unpack2(b, b0, b1);
+    return pack2(lo ? a0 : b0, hi ? a1 : b1);
+}
+
 // One record against the thread's two pixels (Eq. 1).  Returns the weights
 // T alpha (0 where the pixel skips or has stopped) and the transmittances
 // after the record (0 where it has stopped).
@@ -186,11 +194,17 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
                         unpack2(p.T, T0, T1);
                         n_eval += (T0 > 0.f ? 1u : 0u) + (T1 > 0.f ? 1u : 0u);
                     }
+                    const PixelPair before = p;
                     blend_pair(base + off[u], pxf, py0, p, wgt);
                     if (kSave || kCount) {
                         float w0, w1, T0, T1;
                         unpack2(wgt, w0, w1);
                         unpack2(p.T, T0, T1);
+                        if (kSave) {   // an infinite colour reaches only the pixels that composite it
+                            p.C0 = keep2(w0 > 0.f, w1 > 0.f, p.C0, before.C0);
+                            p.C1 = keep2(w0 > 0.f, w1 > 0.f, p.C1, before.C1);
+                            p.C2 = keep2(w0 > 0.f, w1 > 0.f, p.C2, before.C2);
+                        }
                         const uint32_t pos = (uint32_t)(b * kBlendBatch + 1) + off[u] / 16u;
                         if (w0 > 0.f) { Tk0 = T0; last0 = pos; ++n_used; }
                         if (w1 > 0.f) { Tk1 = T1; last1 = pos; ++n_used; }

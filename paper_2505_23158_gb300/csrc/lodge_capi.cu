@@ -2122,7 +2122,7 @@ lodge_status lodge_render_backward(lodge_ctx* ctx, int64_t handle, const float* 
     CUDA_TRY(cudaMemsetAsync(sl.d_small, 0, sizeof(uint32_t) * kSmWords, s));
     launch_blend_bwd(v.cam, v.ranges.as<uint2>(), v.rbits ? v.tkey.as<uint32_t>() : v.tval.as<uint32_t>(),
                      v.rbits ? (1u << v.rbits) - 1u : 0xffffffffu, v.n_keys, v.rec_a.as<float4>(),
-                     v.rec_b.as<float4>(), v.rec_c.as<float>(), v.n_vis, v.T.as<float>(),
+                     v.rec_b.as<float4>(), v.rec_c.as<float>(), v.n_vis, v.rec_rect.as<uint2>(), v.T.as<float>(),
                      v.last.as<uint32_t>(), d_dL_drgb, ws.grec.as<double>(), s);
     launch_project_bwd(v.cam, v.n_vis, v.rec_gid.as<uint32_t>(), ws.grec.as<double>(), v.means,
                        v.act_so.as<float4>(), v.act_q.as<float4>(), v.quats, v.sh, v.sh_degree,
