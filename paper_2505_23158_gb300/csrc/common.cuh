@@ -297,24 +297,18 @@ void launch_digit_scan(uint32_t* hist, int passes, cudaStream_t s);
 void launch_ranges(const uint32_t* tile_key, int64_t n_keys, uint2* ranges, int64_t ntiles,
                    int shift, cudaStream_t s);
 
-// Alpha of a projection record at a pixel (Eq. 1 with the record's
-// Cholesky form): alpha = min(0.99, 2^-((u00 dx + u01 dy)^2 + (u11 dy)^2 -
-// log2 o')), a = (mean', u00, u01), b = (u11, -log2 o', ...).  The
-// compositing thread owns the pixels of rows y and y + 4 of an 8-row block
-// and forms the second row's t and w from the first's by the row step (one
-// FMA each), so a pixel whose row within its tile has bit 2 set takes that
-// form here too: every walk (compositing, adjoint, importance) then decides
-// skip and stop on the same FP32 values.  t and w are returned for the
-// adjoint.
+// Exponent terms of a projection record (Eq. 1 with the record's Cholesky
+// form: alpha = min(0.99, 2^-(t^2 + w^2 - log2 o')), t = u00 dx + u01 dy,
+// w = u11 dy), a = (mean', u00, u01), b = (u11, -log2 o', ...), for the two
+// pixels of one thread: rows py0 (a pixel-centre y) and py0 + 4 of an 8-row
+// block.  The second row's t and w are formed from the first's by the row
+// step (one FMA each).  Every walk (compositing, adjoint, importance) takes
+// this form, so all decide skip and stop on the same FP32 values.
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float alpha_of(float4 b, float t, float w) {
-    return fminf(0.99f, ex2_approx(-fmaf(t, t, fmaf(w, w, b.y))));
-}
-// t and w at row py0 (a pixel-centre y) and at py0 + 4
 __device__ __forceinline__ void row_pair_tw(float4 a, float4 b, float dx, float py0, float& t0, float& w0,
                                             float& t1, float& w1) {
     const float dy = py0 - a.y;
@@ -322,20 +316,6 @@ __device__ __forceinline__ void row_pair_tw(float4 a, float4 b, float dx, float 
     w0 = b.x * dy;
     t1 = fmaf(4.f, a.w, t0);
     w1 = fmaf(4.f, b.x, w0);
-}
-// t and w at pixel row y (image row; tiles start at multiples of 16, so bit
-// 2 of y is bit 2 of the row within the tile)
-__device__ __forceinline__ void pixel_tw(float4 a, float4 b, float dx, int y, float& t, float& w) {
-    float t0, w0, t1, w1;
-    if (y & 4) {
-        row_pair_tw(a, b, dx, (float)(y - 4) + 0.5f, t0, w0, t1, w1);
-        t = t1;
-        w = w1;
-    } else {
-        row_pair_tw(a, b, dx, (float)y + 0.5f, t0, w0, t1, w1);
-        t = t0;
-        w = w0;
-    }
 }
 
 // K7: per tile front-to-back compositing.
@@ -381,6 +361,7 @@ struct BlendFrame {
     float* rgb;
     float* T_final;
     uint32_t* last;
+    uint32_t* rec_score;       // importance walk: largest weight per record (FP32 bits)
 };
 constexpr int kMaxBlendBatch = 64;
 struct BlendBatch {
@@ -403,7 +384,8 @@ void launch_blend_batch(const BlendFrame* frames, int n, cudaStream_t s, uint32_
 void launch_importance(const DevCamera& cam, const uint2* ranges, const uint32_t* tile_val,
                        uint32_t vmask, int64_t n_keys, const float4* rec_a, const float4* rec_b,
                        const float* rec_c, int64_t n_rec, const uint32_t* rec_gid, float* rgb,
-                       uint32_t* rec_score, int64_t n_total, float* score, cudaStream_t s);
+                       uint32_t* rec_score, int64_t n_total, float* score, cudaStream_t s, int bin_log2,
+                       const uint2* rec_rect);
 
 // K8 / K9: adjoint of compositing and projection (fine-tuning path).
 // grec: n_rec x 9 doubles, zeroed: the adjoint sums of each record (k_backward.cu).

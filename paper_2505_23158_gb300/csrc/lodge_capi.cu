@@ -594,12 +594,12 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     const int64_t ptiles = proj_status_words(na);
     TRY(ensure(ctx, ws.status, sizeof(uint32_t) * (size_t)ptiles, s));
     TRY(ensure(ctx, ws.doffs, sizeof(uint32_t) * 8 * 256, s));
-    // frames kept for the adjoint and the importance walk use per-tile lists
-    // (their per-pixel positions index the tile's own list); otherwise the
-    // context's bin size, or by default per-tile lists for active sets of
+    // frames kept for the adjoint use per-tile lists (their per-pixel
+    // positions index the tile's own list); otherwise the context's bin
+    // size, or by default per-tile lists for active sets of
     // kPerTileActiveMin Gaussians or more (many small splats, whose bin
     // lists are long against their tiles' lists) and bins of 2x2 tiles below
-    const int bl = (save || importance) ? 0
+    const int bl = save ? 0
                    : ctx->bin_log2 >= 0 ? ctx->bin_log2
                    : (na >= kPerTileActiveMin ? 0 : 1);
     // the key capacity is learned per bin size
@@ -790,9 +790,10 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     } else if (importance) {
         TRY(ensure(ctx, ws.iscore, sizeof(uint32_t) * nv1, s));
         CUDA_TRY(cudaMemsetAsync(ws.iscore.p, 0, sizeof(uint32_t) * nv1, s));
-        launch_importance(cam, ws.ranges.as<uint2>(), rec_of_pair, vmask, n_keys, ws.rec_a.as<float4>(),
+        launch_importance(cam, ws.ranges.as<uint2>(), rec_of_pair, vmask, n_bkeys, ws.rec_a.as<float4>(),
                           ws.rec_b.as<float4>(), ws.rec_c.as<float>(), n_vis, ws.rec_gid.as<uint32_t>(),
-                          d_rgb, ws.iscore.as<uint32_t>(), dsc.n_total, importance, s);
+                          d_rgb, ws.iscore.as<uint32_t>(), dsc.n_total, importance, s, bl,
+                          ws.rec_rect.as<uint2>());
     } else {
         launch_blend(cam, ws.ranges.as<uint2>(), rec_of_pair, vmask, n_bkeys, ws.rec_a.as<float4>(),
                      ws.rec_b.as<float4>(), ws.rec_c.as<float>(), n_vis, bo, s, bl, ws.rec_rect.as<uint2>(),

@@ -76,6 +76,10 @@ __device__ __forceinline__ float ge01(float a, float b) {
 // One thread tests its record against all four blocks: the reciprocals are
 // the record's, the clamped x terms a column's and the y terms a row's, so
 // that four tests cost about 80 operations instead of 45 each.
+//
+// kNan: a record whose form is not a number (a covariance that overflows
+// FP32) is kept, as in a walk without the test; the plain frames drop it.
+template <bool kNan>
 __device__ __forceinline__ uint32_t blocks_met(const float4 a, const float4 b, const uint2 rect, uint32_t tx0,
                                                uint32_t ty0) {
     constexpr float kLog2_255 = 7.99435343f;
@@ -112,7 +116,7 @@ __device__ __forceinline__ uint32_t blocks_met(const float4 a, const float4 b, c
             const float dx = fminf(fmaxf(xm[r], X0[c]), X1[c]);
             const float t2 = fmaf(u00, dx, uy[r]);
             const float q = fminf(fmaf(t1, t1, w1 * w1), fmaf(t2, t2, wy[r]));
-            if (cx[c] && cy[r] && q <= lim) met |= 1u << (2 * r + c);
+            if (cx[c] && cy[r] && (kNan ? !(q > lim) : q <= lim)) met |= 1u << (2 * r + c);
         }
     return met;
 }

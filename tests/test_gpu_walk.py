@@ -98,3 +98,27 @@ def test_gradients_of_list_lengths(env, n, wh):
     touched = (grads(alone)[4].abs().sum(1) > 0)          # records that pixel (0, 0) composites
     hurt = ~torch.isfinite(grads(w)[4]).all(1)
     assert not (hurt & ~touched).any()
+
+
+@pytest.mark.parametrize("n,wh", [(1, (8, 8)), (3, (16, 16)), (4, (7, 9)), (127, (15, 16)), (128, (33, 16)),
+                                  (129, (16, 40)), (300, (9, 23))])
+def test_importance_of_list_lengths(env, n, wh):
+    """The scoring walk on the same stacks: every score within 2e-4 of the
+    oracle's bracket (the bar of the importance tests), and the same for
+    every bin size, whose lists hold the same records in the same order."""
+    torch, api, ctx = env
+    scene = _stack_scene(n, 90 + n, opacity=-1.0)
+    cam = synth.look_at((0.0, 0.0, -3.0), (0.0, 0.0, 1.0), (0.0, -1.0, 0.0), wh[0], wh[1], 30.0)
+    ref, clean = O.importance(O.OracleScene(scene), cam, np.arange(n))
+    sid = ctx.load_scene(scene)
+    try:
+        scores = []
+        for log2 in (0, 1, 3):
+            ctx.set_bin_size(log2)
+            scores.append(ctx.importance(sid, api.FULL, [cam]))
+            s = scores[-1].cpu().numpy().astype(np.float64)
+            assert (s >= np.minimum(clean, ref) - 2e-4).all() and (s <= ref + 2e-4).all()
+            assert torch.equal(scores[-1], scores[0])
+    finally:
+        ctx.set_bin_size(-1)
+        ctx.unload_scene(sid)
