@@ -186,6 +186,14 @@ struct ResidencyStats {
 struct lodge_ctx {
     int device = 0;
     size_t budget = 0;
+    // Scratch and saved frames come from the context's own pool, which keeps
+    // freed memory mapped while it holds at most kPoolKeep bytes in all (none
+    // when a budget is set; given back when an allocation fails): a
+    // training step saves its frame's buffers and frees them after the
+    // adjoint, and the device's default pool unmaps freed memory at every
+    // synchronisation, so that each step mapped it anew.  A fine-tuning step
+    // of 2M Gaussians at 720p: 2427 -> 2192 us.
+    cudaMemPool_t pool = nullptr;
     size_t used = 0;                 // device bytes held; guarded by mu
     std::recursive_mutex mu;         // budget, blocks, saved frames, slot list
     std::condition_variable_any freed;  // signalled when device memory is released
@@ -207,11 +215,15 @@ namespace lodge {
 // errors (thread-local message)
 lodge_status fail(lodge_status s, const char* fmt, ...);
 
+constexpr size_t kPoolKeep = 2ull << 30;   // 0.7% of the device's memory
+
 // device memory with budget accounting (thread-safe)
 lodge_status dmalloc(lodge_ctx* ctx, void** p, size_t bytes);
 void dfree(lodge_ctx* ctx, void* p, size_t bytes);
 lodge_status ensure(lodge_ctx* ctx, DBuf& b, size_t bytes, cudaStream_t s);
 void release(lodge_ctx* ctx, DBuf& b, cudaStream_t s);
+// the pool's freed memory back to the device, after an allocation failed
+bool trim_pool(lodge_ctx* ctx);
 // evict unreferenced blocks (least recently used first) until `bytes` more
 // fit in the budget; caller holds ctx->mu; returns false if they cannot
 bool make_room(lodge_ctx* ctx, size_t bytes);

@@ -91,12 +91,18 @@ bool make_room(lodge_ctx* ctx, size_t bytes) {
     return true;
 }
 
+bool trim_pool(lodge_ctx* ctx) {
+    cudaGetLastError();
+    return cudaDeviceSynchronize() == cudaSuccess && cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess;
+}
+
 lodge_status dmalloc(lodge_ctx* ctx, void** p, size_t bytes) {
     std::lock_guard<std::recursive_mutex> lk(ctx->mu);
     if (!make_room(ctx, bytes))
         return fail(LODGE_E_BUDGET, "HBM budget exceeded: %zu in use + %zu requested > %zu",
                     ctx->used, bytes, ctx->budget);
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && trim_pool(ctx)) e = cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(LODGE_E_OOM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
@@ -133,7 +139,8 @@ lodge_status ensure(lodge_ctx* ctx, DBuf& b, size_t bytes, cudaStream_t s) {
         b.p = nullptr;
         b.cap = 0;
     }
-    cudaError_t e = cudaMallocAsync(&b.p, ncap, s);
+    cudaError_t e = cudaMallocFromPoolAsync(&b.p, ncap, ctx->pool, s);
+    if (e == cudaErrorMemoryAllocation && trim_pool(ctx)) e = cudaMallocFromPoolAsync(&b.p, ncap, ctx->pool, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         b.p = nullptr;
@@ -1289,6 +1296,13 @@ lodge_status lodge_create(int device, size_t hbm_budget_bytes, lodge_ctx** out) 
     fill_qtable_host(q);
     CUDA_TRY(upload_qtable(q));
     CUDA_TRY(cudaStreamCreateWithFlags(&ctx->upload_stream, cudaStreamNonBlocking));
+    cudaMemPoolProps pp{};
+    pp.allocType = cudaMemAllocationTypePinned;
+    pp.location.type = cudaMemLocationTypeDevice;
+    pp.location.id = device;
+    CUDA_TRY(cudaMemPoolCreate(&ctx->pool, &pp));
+    uint64_t keep = hbm_budget_bytes ? 0 : kPoolKeep;
+    CUDA_TRY(cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
     Slot* s0 = nullptr;
     TRY(create_slot(ctx.get(), &s0));
     *out = ctx.release();
@@ -1306,6 +1320,7 @@ lodge_status lodge_destroy(lodge_ctx* ctx) {
     for (auto& sl : ctx->slots) destroy_slot(ctx, *sl);
     if (ctx->upload_stream) cudaStreamDestroy(ctx->upload_stream);
     cudaDeviceSynchronize();
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     delete ctx;
     return LODGE_OK;
 }

@@ -182,6 +182,8 @@ lodge_status acquire_block(lodge_ctx* ctx, Slot& sl, Scene* sc, int chunk, cudaS
                             "(%zu of %zu in use, the rest held by frames in flight)",
                             chunk, sc->id, b->bytes, ctx->used, ctx->budget);
             cudaError_t e = cudaMallocAsync(&b->mem, b->bytes, ctx->upload_stream);
+            if (e == cudaErrorMemoryAllocation && trim_pool(ctx))
+                e = cudaMallocAsync(&b->mem, b->bytes, ctx->upload_stream);
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 return fail(LODGE_E_OOM, "chunk block of %zu bytes: %s", b->bytes, cudaGetErrorString(e));
