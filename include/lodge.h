@@ -328,7 +328,7 @@ lodge_status lodge_render_params(lodge_ctx* ctx, int64_t n, const float* d_means
  *   num_levels: 1 .. 8, finest first; level_n (host, num_levels): sizes.
  *   d_means .. d_sh (host arrays of num_levels DEVICE pointers, caller-owned,
  *     layouts as lodge_level_desc; SH 16-byte aligned); activated on the
- *     device in FP32 into one gid-ordered store (gid = index into the levels
+ *     device in FP32 as they are read (gid = index into the levels
  *     concatenated finest first).
  *   filter_var (host, num_levels): the Eq. 3 variance of each level.
  *   d_inner (host, num_levels - 1, ascending, metres): this frame's

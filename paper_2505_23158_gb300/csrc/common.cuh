@@ -198,10 +198,23 @@ struct ProjSources {
     const uint32_t* gid_b = nullptr;
     int64_t n_a = 0, n_b = 0, npad_a = 0, npad_b = 0;
 };
+// Attribute source of a parameter frame: the caller's raw arrays, level by
+// level (device pointers; gid = index into the levels concatenated, bounds in
+// the scene's level_off).  Activated as they are read; a frame kept for the
+// adjoint also stores its records' activated attributes.
+struct RawLevels {
+    const float* means[kMaxLevels] = {nullptr};       // n x 3
+    const float* log_scales[kMaxLevels] = {nullptr};  // n x 3
+    const float* quats[kMaxLevels] = {nullptr};       // n x 4
+    const float* logits[kMaxLevels] = {nullptr};
+    const float4* sh[kMaxLevels] = {nullptr};         // n x 48 floats
+    float4* rec_so = nullptr;                         // per record: (s0, s1, s2, opacity)
+    float4* rec_q = nullptr;                          // per record: unit quaternion
+};
 void launch_project(const DevScene& sc, const DevCamera& cam, const uint32_t* list,
                     int64_t n_active, float tA, float tB, const ProjectOut& o, uint32_t* status,
                     uint32_t* tile_counter, uint32_t* err, cudaStream_t s,
-                    const ProjSources* src = nullptr);
+                    const ProjSources* src = nullptr, const RawLevels* raw = nullptr);
 // copy the extent table to this device's constant memory (once per device)
 cudaError_t upload_qtable(const float* q65);
 
@@ -397,7 +410,7 @@ void launch_blend_bwd(const DevCamera& cam, const uint2* ranges, const uint32_t*
 // variance of each level (gid ranges level_off) and the trained level's gid
 // range [train_lo, train_hi).  Records outside it get no gradient; the raw
 // parameter and gradient arrays hold the trained level only and are indexed
-// by gid - train_lo (the activated arrays by gid).
+// by gid - train_lo (the activated arrays by record).
 struct BwdLevels {
     int32_t num_levels = 1;
     int64_t level_off[kMaxLevels + 1] = {0};

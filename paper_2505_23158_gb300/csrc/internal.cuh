@@ -80,7 +80,7 @@ struct Saved {
                 *sh = nullptr;
     int sh_degree = 3;
     BwdLevels lv;            // levels, filter variances and the trained level's gid range
-    DBuf act_so, act_q;
+    DBuf act_so, act_q;      // per record: activated (scale, opacity) and quaternion
 };
 
 struct Workspace {

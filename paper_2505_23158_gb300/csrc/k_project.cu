@@ -25,7 +25,22 @@ struct ProjParams {
     float tA, tB;
     ProjectOut o;
     ProjSources src;        // block sources (kBlocks only)
+    RawLevels raw;          // raw parameters (kRaw only)
 };
+
+// where an entry's attributes come from
+enum : int { kStore = 0, kBlocks = 1, kRaw = 2 };
+
+// FP32 activation of Gaussian r of level l of the raw parameters
+__device__ __forceinline__ void activate(const RawLevels& raw, int l, int64_t r, float4& so, float4& q) {
+    const float* ls = raw.log_scales[l] + 3 * r;
+    const float* qr = raw.quats[l] + 4 * r;
+    const float s0 = ls[0], s1 = ls[1], s2 = ls[2], lg = raw.logits[l][r];
+    const float w = qr[0], x = qr[1], y = qr[2], z = qr[3];
+    so = make_float4(expf(s0), expf(s1), expf(s2), 1.f / (1.f + expf(-lg)));
+    const float n = rsqrtf(w * w + x * x + y * y + z * z);
+    q = make_float4(w * n, x * n, y * n, z * n);
+}
 
 __device__ __forceinline__ float fm(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fa(float a, float b) { return __fadd_rn(a, b); }
@@ -180,7 +195,13 @@ __device__ __forceinline__ bool key_splat(const DevScene& sc, const DevCamera& c
 // six CTAs per SM (at most 42 registers): the kernel is bound by the
 // latency of its dependent gathers, so resident warps matter more than the
 // few spilled words
-template <bool kBlocks>
+//
+// kRaw reads the caller's parameter arrays where they lie.  Activating them
+// into a store first (a transpose of the 192-byte SH rows above all, of every
+// Gaussian, seen or not) moved 472 bytes a Gaussian: 160 us of launches
+// before a projection of 110 us for 2M Gaussians, 58% of them visible; this
+// one takes 135 us alone.
+template <int kSrc>
 __global__ void __launch_bounds__(kProjThreads, 6)
 project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict__ tile_counter,
                uint32_t* __restrict__ err) {
@@ -213,13 +234,15 @@ project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict
     const float4* sq = sc.quat;
     const float4* ssh = sc.sh;
     int64_t npad = P.n_pad;
+    int lvl = 0;          // kRaw: the entry's level and its index there
+    int64_t at = 0;
     if (i < P.n_active) {
         uint32_t e = P.list ? P.list[i] : (uint32_t)i;
         idx = e & kGidMask;
         float mult = 1.f;
         if ((e & kFlagA) && !(e & kFlagB)) mult = P.tA;
         else if ((e & kFlagB) && !(e & kFlagA)) mult = P.tB;
-        if (kBlocks) {
+        if (kSrc == kBlocks) {
             const bool fa = (e & kFlagA) != 0;
             const int64_t nb = fa ? P.src.n_a : P.src.n_b;
             if ((int64_t)idx >= nb) { atomicOr(err, kErrBadIndex); idx = 0; mult = 0.f; }
@@ -237,8 +260,19 @@ project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict
         }
         // the mean, (scale, opacity) and quaternion are loaded together, so
         // that one memory latency, not three in a row, precedes the key spec
-        const float mxw = smx[idx], myw = smy[idx], mzw = smz[idx];
-        const float4 so = sso[idx], qq = sq[idx];
+        float mxw, myw, mzw;
+        float4 so, qq;
+        if (kSrc == kRaw) {
+            while (lvl + 1 < sc.num_levels && (int64_t)g >= sc.level_off[lvl + 1]) ++lvl;
+            at = (int64_t)g - sc.level_off[lvl];
+            const float* m = P.raw.means[lvl] + 3 * at;
+            mxw = m[0]; myw = m[1]; mzw = m[2];
+            activate(P.raw, lvl, at, so, qq);
+        } else {
+            mxw = smx[idx]; myw = smy[idx]; mzw = smz[idx];
+            so = sso[idx];
+            qq = sq[idx];
+        }
         KeySplat ks;
         vis = key_splat<true>(sc, cam, mxw, myw, mzw, sso, sq, idx, g, mult, ks, so, qq);
         d0 = ks.d0; d1 = ks.d1; d2 = ks.d2;
@@ -246,8 +280,14 @@ project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict
             // start the SH planes' way into L2 now: the block scan and the
             // conic come before they are read
             const int npl = (3 * (sc.sh_degree + 1) * (sc.sh_degree + 1) + 3) / 4;
-            for (int j = 0; j < npl; ++j)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(ssh + (int64_t)j * npad + idx));
+            if (kSrc == kRaw) {   // a row: one or two 128-byte lines
+                const float4* row = P.raw.sh[lvl] + 12 * at;
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(row));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(row + npl - 1));
+            } else {
+                for (int j = 0; j < npl; ++j)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(ssh + (int64_t)j * npad + idx));
+            }
         }
         if (vis) {
             z = ks.z; mxp = ks.mx; myp = ks.my; o = ks.op;
@@ -321,7 +361,7 @@ project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict
 #pragma unroll
         for (int j = 0; j < 12; ++j) {
             if (4 * j >= nf) break;
-            float4 v4 = __ldcs(ssh + (int64_t)j * npad + idx);
+            const float4 v4 = kSrc == kRaw ? __ldg(P.raw.sh[lvl] + 12 * at + j) : __ldcs(ssh + (int64_t)j * npad + idx);
             float vv[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
             for (int cc = 0; cc < 4; ++cc) {
@@ -363,6 +403,12 @@ project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict
     P.o.rec_gid[pos] = g;
     P.o.depth_key[pos] = __float_as_uint(z);
     P.o.depth_val[pos] = pos;
+    if (kSrc == kRaw && P.raw.rec_so) {   // read again: holding them through the kernel costs registers
+        float4 so, q;
+        activate(P.raw, lvl, at, so, q);
+        P.raw.rec_so[pos] = so;
+        P.raw.rec_q[pos] = q;
+    }
 }
 
 
@@ -434,7 +480,7 @@ cudaError_t upload_qtable(const float* q65) {
 void launch_project(const DevScene& sc, const DevCamera& cam, const uint32_t* list,
                     int64_t n_active, float tA, float tB, const ProjectOut& o, uint32_t* status,
                     uint32_t* tile_counter, uint32_t* err, cudaStream_t s,
-                    const ProjSources* src) {
+                    const ProjSources* src, const RawLevels* raw) {
     ProjParams P;
     P.sc = sc;
     P.cam = cam;
@@ -445,12 +491,15 @@ void launch_project(const DevScene& sc, const DevCamera& cam, const uint32_t* li
     P.tB = tB;
     P.o = o;
     if (src) P.src = *src;
+    if (raw) P.raw = *raw;
     int64_t ntiles = (n_active + kProjThreads - 1) / kProjThreads;
     if (ntiles == 0) return;
-    if (src)
-        project_kernel<true><<<(unsigned)ntiles, kProjThreads, 0, s>>>(P, status, tile_counter, err);
+    if (raw)
+        project_kernel<kRaw><<<(unsigned)ntiles, kProjThreads, 0, s>>>(P, status, tile_counter, err);
+    else if (src)
+        project_kernel<kBlocks><<<(unsigned)ntiles, kProjThreads, 0, s>>>(P, status, tile_counter, err);
     else
-        project_kernel<false><<<(unsigned)ntiles, kProjThreads, 0, s>>>(P, status, tile_counter, err);
+        project_kernel<kStore><<<(unsigned)ntiles, kProjThreads, 0, s>>>(P, status, tile_counter, err);
 }
 
 size_t threshold_cost_smem(int K) { return sizeof(unsigned long long) * (2 * K + 2) + sizeof(float) * K; }

@@ -403,6 +403,7 @@ struct Active {
     double tA = 1.0, tB = 1.0;
     bool blocks = false;       // entries index into chunk blocks (streamed scenes)
     ProjSources src;
+    const RawLevels* raw = nullptr;   // parameter frames: the caller's arrays
 };
 
 static lodge_status select_streamed(lodge_ctx* ctx, Slot& sl, Scene* sc, lodge_mode mode,
@@ -662,10 +663,20 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     // depth sort's (from K3)
     po.depth_hist = ws.doffs.as<uint32_t>() + 4 * 256;
     po.bin_log2 = bl;
+    RawLevels raw;
+    if (act.raw) {
+        raw = *act.raw;
+        if (save) {   // the adjoint's view of the records
+            TRY(ensure(ctx, ws.act_so, sizeof(float4) * na1, s));
+            TRY(ensure(ctx, ws.act_q, sizeof(float4) * na1, s));
+            raw.rec_so = ws.act_so.as<float4>();
+            raw.rec_q = ws.act_q.as<float4>();
+        }
+    }
     prof_begin(sl, LODGE_STAGE_PROJECT, s);
     launch_project(dsc, cam, act.list, na, (float)act.tA, (float)act.tB, po,
                    ws.status.as<uint32_t>(), sl.d_small + kSmCtrProj, sl.d_small + kSmErr, s,
-                   act.blocks ? &act.src : nullptr);
+                   act.blocks ? &act.src : nullptr, act.raw ? &raw : nullptr);
     // (the launch count of the projection stage includes the frame's fill)
     prof_end(sl, LODGE_STAGE_PROJECT, s, (na > 0 ? 1 : 0) + (deferred ? 1 : 0));
     CUDA_TRY(cudaGetLastError());
@@ -883,6 +894,10 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
         take(save->ranges, ws.ranges);
         take(save->T, ws.T);
         take(save->last, ws.last);
+        if (act.raw) {
+            take(save->act_so, ws.act_so);
+            take(save->act_q, ws.act_q);
+        }
     }
     return LODGE_OK;
 }
@@ -1132,28 +1147,7 @@ __global__ void debug_records_kernel(int64_t n, const float4* ra, const float4* 
     if (rgb) { rgb[3 * i] = b.z; rgb[3 * i + 1] = b.w; rgb[3 * i + 2] = rc[i]; }
 }
 
-// FP32 device activation for the raw-parameter path.
-__global__ void activate_kernel(int64_t n, const float* ls, const float* q, const float* lg,
-                                float4* so, float4* qo) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s0 = expf(ls[3 * i]), s1 = expf(ls[3 * i + 1]), s2 = expf(ls[3 * i + 2]);
-    float o = 1.f / (1.f + expf(-lg[i]));
-    so[i] = make_float4(s0, s1, s2, o);
-    float w = q[4 * i], x = q[4 * i + 1], y = q[4 * i + 2], z = q[4 * i + 3];
-    float r = rsqrtf(w * w + x * x + y * y + z * z);
-    qo[i] = make_float4(w * r, x * r, y * r, z * r);
-}
-
-// N x 48 SH coefficients -> 12 planes of float4 with stride np
-__global__ void sh_planes_kernel(int64_t n, const float* sh, float4* planes, int64_t np) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float4* src = reinterpret_cast<const float4*>(sh + 48 * i);
-#pragma unroll
-    for (int j = 0; j < 12; ++j) planes[(size_t)j * np + i] = src[j];
-}
-
+// N x 3 means -> planes, for the level selection of a parameter frame
 __global__ void planes_kernel(int64_t n, const float* means, float* mx, float* my, float* mz) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -1960,21 +1954,6 @@ lodge_status lodge_render_params(lodge_ctx* ctx, int64_t n, const float* d_means
     CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Slot& sl = *ctx->slots[0];
-    Workspace& ws = sl.ws;
-    const size_t n1 = (size_t)std::max<int64_t>(n, 1);
-    const int64_t NP = std::max<int64_t>((n + 63) / 64 * 64, 64);
-    TRY(ensure(ctx, ws.act_so, sizeof(float4) * n1, s));
-    TRY(ensure(ctx, ws.act_q, sizeof(float4) * n1, s));
-    TRY(ensure(ctx, ws.mtmp, sizeof(float) * 3 * (size_t)NP + sizeof(float4) * 12 * (size_t)NP, s));
-    float* mp = ws.mtmp.as<float>();
-    float4* shp = reinterpret_cast<float4*>(mp + 3 * NP);
-    if (n) {
-        unsigned nb = (unsigned)((n + 255) / 256);
-        activate_kernel<<<nb, 256, 0, s>>>(n, d_log_scales, d_quats, d_opacity_logits, ws.act_so.as<float4>(), ws.act_q.as<float4>());
-        planes_kernel<<<nb, 256, 0, s>>>(n, d_means, mp, mp + NP, mp + 2 * NP);
-        sh_planes_kernel<<<nb, 256, 0, s>>>(n, d_sh, shp, NP);
-        CUDA_TRY(cudaGetLastError());
-    }
     DevScene d;
     d.n_total = n;
     d.num_levels = 1;
@@ -1982,12 +1961,15 @@ lodge_status lodge_render_params(lodge_ctx* ctx, int64_t n, const float* d_means
     d.level_off[0] = 0;
     for (int l = 1; l <= kMaxLevels; ++l) d.level_off[l] = n;
     d.filter_var[0] = filter_var;
-    d.mx = mp; d.my = mp + NP; d.mz = mp + 2 * NP;
-    d.scale_op = ws.act_so.as<float4>();
-    d.quat = ws.act_q.as<float4>();
-    d.sh = shp;
+    RawLevels raw;
+    raw.means[0] = d_means;
+    raw.log_scales[0] = d_log_scales;
+    raw.quats[0] = d_quats;
+    raw.logits[0] = d_opacity_logits;
+    raw.sh[0] = reinterpret_cast<const float4*>(d_sh);
     Active act;
     act.n = n;
+    act.raw = &raw;
     std::unique_ptr<Saved> sv;
     if (save_for_backward) sv.reset(new Saved());
     TRY(render_frame(ctx, sl, d, act, *cam, d_rgb, s, sv.get(), stats, true));
@@ -2002,8 +1984,6 @@ lodge_status lodge_render_params(lodge_ctx* ctx, int64_t n, const float* d_means
         sv->lv.filter_var[0] = filter_var;
         sv->lv.train_lo = 0;
         sv->lv.train_hi = n;
-        take(sv->act_so, ws.act_so);
-        take(sv->act_q, ws.act_q);
         std::lock_guard<std::recursive_mutex> lk(ctx->mu);
         int64_t h = ctx->next_handle++;
         ctx->saved[h] = std::move(sv);
@@ -2059,35 +2039,35 @@ lodge_status lodge_render_params_lod(lodge_ctx* ctx, int32_t num_levels, const i
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Slot& sl = *ctx->slots[0];
     Workspace& ws = sl.ws;
-    const size_t n1 = (size_t)std::max<int64_t>(n, 1);
+    // the selection reads the means as planes; all else is read in place
     const int64_t NP = std::max<int64_t>((n + 63) / 64 * 64, 64);
-    TRY(ensure(ctx, ws.act_so, sizeof(float4) * n1, s));
-    TRY(ensure(ctx, ws.act_q, sizeof(float4) * n1, s));
-    TRY(ensure(ctx, ws.mtmp, sizeof(float) * 3 * (size_t)NP + sizeof(float4) * 12 * (size_t)NP, s));
-    float* mp = ws.mtmp.as<float>();
-    float4* shp = reinterpret_cast<float4*>(mp + 3 * NP);
+    RawLevels raw;
+    float* mp = nullptr;
+    if (num_levels > 1) {
+        TRY(ensure(ctx, ws.mtmp, sizeof(float) * 3 * (size_t)NP, s));
+        mp = ws.mtmp.as<float>();
+    }
     for (int l = 0; l < num_levels; ++l) {
         const int64_t nl = level_n[l], o = off[l];
-        if (!nl) continue;
-        unsigned nb = (unsigned)((nl + 255) / 256);
-        activate_kernel<<<nb, 256, 0, s>>>(nl, d_log_scales[l], d_quats[l], d_opacity_logits[l],
-                                           ws.act_so.as<float4>() + o, ws.act_q.as<float4>() + o);
-        planes_kernel<<<nb, 256, 0, s>>>(nl, d_means[l], mp + o, mp + NP + o, mp + 2 * NP + o);
-        sh_planes_kernel<<<nb, 256, 0, s>>>(nl, d_sh[l], shp + o, NP);
-        CUDA_TRY(cudaGetLastError());
+        raw.means[l] = d_means[l];
+        raw.log_scales[l] = d_log_scales[l];
+        raw.quats[l] = d_quats[l];
+        raw.logits[l] = d_opacity_logits[l];
+        raw.sh[l] = reinterpret_cast<const float4*>(d_sh[l]);
+        if (nl && mp)
+            planes_kernel<<<(unsigned)((nl + 255) / 256), 256, 0, s>>>(nl, d_means[l], mp + o, mp + NP + o,
+                                                                       mp + 2 * NP + o);
     }
+    CUDA_TRY(cudaGetLastError());
     DevScene d;
     d.n_total = n;
     d.num_levels = num_levels;
     d.sh_degree = sh_degree;
     for (int l = 0; l <= kMaxLevels; ++l) d.level_off[l] = off[l];
     for (int l = 0; l < num_levels; ++l) d.filter_var[l] = filter_var[l];
-    d.mx = mp; d.my = mp + NP; d.mz = mp + 2 * NP;
-    d.scale_op = ws.act_so.as<float4>();
-    d.quat = ws.act_q.as<float4>();
-    d.sh = shp;
     Active act;
     if (num_levels > 1) {
+        d.mx = mp; d.my = mp + NP; d.mz = mp + 2 * NP;
         int64_t na = 0;
         TRY(run_lod_select(ctx, sl, d, cam->center, d_inner, s, &na));
         act.list = ws.list.as<uint32_t>();
@@ -2095,6 +2075,7 @@ lodge_status lodge_render_params_lod(lodge_ctx* ctx, int32_t num_levels, const i
     } else {
         act.n = n;
     }
+    act.raw = &raw;
     std::unique_ptr<Saved> sv;
     if (save_for_backward) sv.reset(new Saved());
     TRY(render_frame(ctx, sl, d, act, *cam, d_rgb, s, sv.get(), stats, true, d_score));
@@ -2110,8 +2091,6 @@ lodge_status lodge_render_params_lod(lodge_ctx* ctx, int32_t num_levels, const i
         for (int l = 0; l < num_levels; ++l) sv->lv.filter_var[l] = filter_var[l];
         sv->lv.train_lo = off[tl];
         sv->lv.train_hi = off[tl + 1];
-        take(sv->act_so, ws.act_so);
-        take(sv->act_q, ws.act_q);
         std::lock_guard<std::recursive_mutex> lk(ctx->mu);
         int64_t h = ctx->next_handle++;
         ctx->saved[h] = std::move(sv);
