@@ -24,6 +24,37 @@ constexpr uint32_t kSpinLimit = 1u << 22;   // iterations before a wait gives up
 constexpr uint32_t kSpinFast = 64;          // polls before a wait starts to sleep between polls
 
 // ---------------------------------------------------------------------------
+// chained launches: the kernels of a lone frame follow one another on one
+// stream, each too short to hide the next one's launch.  Launched chained, a
+// kernel's CTAs start as soon as every CTA of the one before has started and
+// there is room, and wait at chain_wait until that kernel has completed with
+// its writes visible (as it waited for its own predecessor, so has everything
+// before).  Every kernel of the chain calls chain_wait before it touches
+// global memory.  Both calls do nothing in a launch that is not chained.
+// Frames that share the SMs with other streams' frames are not chained: a
+// waiting CTA holds room that the other frames' kernels use.
+// A lone 1080p chunk frame 310 -> 288 us, an LOD frame 305 -> 291, 256 x 256
+// of 4,096 Gaussians 136 -> 128 (eleven launches each).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+inline void launch_chained(bool chained, void (*kernel)(P...), unsigned grid, unsigned threads, cudaStream_t s,
+                           A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = chained ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, P(args)...);   // an error stays for the caller's cudaGetLastError
+}
+
+// ---------------------------------------------------------------------------
 // decoupled look-back over 32-bit status words: flag in bits 31..30, value in
 // bits 29..0 (so per-tile counts must stay below 2^30).
 // ---------------------------------------------------------------------------
@@ -214,7 +245,7 @@ struct RawLevels {
 void launch_project(const DevScene& sc, const DevCamera& cam, const uint32_t* list,
                     int64_t n_active, float tA, float tB, const ProjectOut& o, uint32_t* status,
                     uint32_t* tile_counter, uint32_t* err, cudaStream_t s,
-                    const ProjSources* src = nullptr, const RawLevels* raw = nullptr);
+                    const ProjSources* src = nullptr, const RawLevels* raw = nullptr, bool chained = false);
 // copy the extent table to this device's constant memory (once per device)
 cudaError_t upload_qtable(const float* q65);
 
@@ -267,7 +298,7 @@ int launch_onesweep(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t
                     const uint32_t* digit_offsets = nullptr, bool final_keys = true, int shift0 = 0,
                     uint2* ranges = nullptr, uint32_t range_tiles = 0,
                     const unsigned long long* d_count = nullptr, bool scratch_cleared = false,
-                    bool digit_counts = false);
+                    bool digit_counts = false, bool chained = false);
 int onesweep_launches(int64_t n, int key_bits, bool offsets_supplied);
 
 // K4: emit (bin, record) pairs in depth order.  A bin is a square of
@@ -299,7 +330,7 @@ int launch_emit_counted(const uint32_t* sorted_rec, int64_t n_vis_cap, const uns
                          const uint2* rec_rect, int32_t bins_x, int bin_log2, int64_t key_cap,
                          const unsigned long long* d_nkeys, uint32_t* tile_key, uint32_t* tile_val,
                          int rbits, int key_bits, uint32_t* digit_hist, uint32_t* status,
-                         uint32_t* tile_counter, uint32_t* err, cudaStream_t s);
+                         uint32_t* tile_counter, uint32_t* err, cudaStream_t s, bool chained = false);
 
 int emit_launches(int64_t n_vis, int64_t n_keys, int bin_log2);
 // exclusive scan, in place, of `passes` 256-bin digit histograms (one launch)
@@ -347,7 +378,7 @@ void launch_blend(const DevCamera& cam, const uint2* ranges, const uint32_t* til
                   int64_t n_keys, const float4* rec_a, const float4* rec_b, const float* rec_c,
                   int64_t n_rec, const BlendOut& o, cudaStream_t s, int bin_log2,
                   const uint2* rec_rect, unsigned long long* pairs = nullptr,
-                  uint32_t* tile_ctr = nullptr);
+                  uint32_t* tile_ctr = nullptr, bool chained = false);
 // tile_ctr (a zeroed device word) makes the compositing a grid of
 // kBlendCtasPerSM CTAs per SM that take tiles from the counter, so that
 // other streams' kernels keep room on every SM while it runs (used when

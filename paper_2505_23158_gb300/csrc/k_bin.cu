@@ -237,6 +237,7 @@ emit_fused_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis,
                   uint32_t* __restrict__ status, uint32_t* __restrict__ counter,
                   uint32_t* __restrict__ err, const unsigned long long* __restrict__ d_nvis,
                   const unsigned long long* __restrict__ d_nkeys) {
+    chain_wait();
     // with device counts, n_vis and n_keys are capacities: the counts decide
     // which CTAs work and the keys must fit n_keys
     if (d_nvis) {
@@ -383,6 +384,7 @@ emit_count_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
                   int bin_log2, uint32_t* __restrict__ tile_sum, uint32_t* __restrict__ err) {
     constexpr int kEmitTileRecs = kEmitThreads * kEmitRecs;
     __shared__ uint32_t s_part[kEmitThreads / 32];
+    chain_wait();
     const int64_t n_vis = device_count(n_vis_cap, d_nvis);
     const int64_t t0 = (int64_t)blockIdx.x * kEmitTileRecs;
     if (t0 >= n_vis) return;   // past the device count (later tiles too)
@@ -413,6 +415,7 @@ __global__ void __launch_bounds__(1024)
 emit_scan_kernel(int tile_recs, uint32_t* __restrict__ tile_sum, int64_t n_vis_cap, const unsigned long long* __restrict__ d_nvis,
                  int64_t key_cap, const unsigned long long* __restrict__ d_nkeys, uint32_t* __restrict__ err) {
     __shared__ uint32_t s_scan[33];
+    chain_wait();
     const int64_t n_vis = device_count(n_vis_cap, d_nvis);
     const int64_t ntiles = (n_vis + tile_recs - 1) / tile_recs;
     uint64_t carry = 0;
@@ -443,6 +446,7 @@ emit_write_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
     __shared__ uint32_t s_big[kEmitTileRecs];     // (thread << 2 | j) of records with many keys
     __shared__ uint32_t s_off[kEmitTileRecs];
     __shared__ uint32_t s_hist[3][256];
+    chain_wait();
     const int64_t n_vis = device_count(n_vis_cap, d_nvis);
     const int64_t t0 = (int64_t)blockIdx.x * kEmitTileRecs;
     if (t0 >= n_vis) return;
@@ -605,7 +609,7 @@ int launch_emit_counted(const uint32_t* sorted_rec, int64_t n_vis_cap, const uns
                         const uint2* rec_rect, int32_t bins_x, int bin_log2, int64_t key_cap,
                         const unsigned long long* d_nkeys, uint32_t* tile_key, uint32_t* tile_val,
                         int rbits, int key_bits, uint32_t* digit_hist, uint32_t* status,
-                        uint32_t* tile_counter, uint32_t* err, cudaStream_t s) {
+                        uint32_t* tile_counter, uint32_t* err, cudaStream_t s, bool chained) {
     const int64_t nb = (n_vis_cap + kEmitThreads - 1) / kEmitThreads;
     if (nb == 0) return 0;
     const int P = (key_bits + 7) / 8;
@@ -615,15 +619,15 @@ int launch_emit_counted(const uint32_t* sorted_rec, int64_t n_vis_cap, const uns
         // count, scan, write (the tile counts and offsets live in `status`,
         // which holds one word per 256 records)
         const unsigned nt = (unsigned)((n_vis_cap + 4 * kEmitThreads - 1) / (4 * kEmitThreads));
-        emit_count_kernel<4><<<nt, kEmitThreads, 0, s>>>(sorted_rec, n_vis_cap, d_nvis, rec_rect, bin_log2,
+        launch_chained(chained, emit_count_kernel<4>, nt, kEmitThreads, s, sorted_rec, n_vis_cap, d_nvis, rec_rect, bin_log2,
                                                          status, err);
-        emit_scan_kernel<<<1, 1024, 0, s>>>(4 * kEmitThreads, status, n_vis_cap, d_nvis, key_cap, d_nkeys, err);
-        emit_write_kernel<4><<<nt, kEmitThreads, 0, s>>>(sorted_rec, n_vis_cap, d_nvis, rec_rect, bin_log2, bins_x,
+        launch_chained(chained, emit_scan_kernel, 1, 1024, s, 4 * kEmitThreads, status, n_vis_cap, d_nvis, key_cap, d_nkeys, err);
+        launch_chained(chained, emit_write_kernel<4>, nt, kEmitThreads, s, sorted_rec, n_vis_cap, d_nvis, rec_rect, bin_log2, bins_x,
                                                          key_cap, status, tile_key, tile_val, rbits, P, last_mask,
                                                          digit_hist, err);
         return 3;
     }
-    emit_fused_kernel<<<(unsigned)nb, kEmitThreads, 0, s>>>(sorted_rec, n_vis_cap, rec_rect, bin_log2, bins_x,
+    launch_chained(chained, emit_fused_kernel, (unsigned)nb, kEmitThreads, s, sorted_rec, n_vis_cap, rec_rect, bin_log2, bins_x,
                                                             key_cap, tile_key, tile_val, rbits, P, last_mask,
                                                             digit_hist, status, tile_counter, err, d_nvis,
                                                             d_nkeys);

@@ -272,6 +272,7 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
 
 template <bool kSave, bool kCount>
 __global__ void __launch_bounds__(kBlendThreads, 8) blend_kernel(BlendFrame f) {
+    chain_wait();
     blend_tile<kSave, kCount>(f, blockIdx.x);
 }
 
@@ -381,7 +382,7 @@ BlendFrame blend_frame(const DevCamera& cam, const uint2* ranges, const uint32_t
 void launch_blend(const DevCamera& cam, const uint2* ranges, const uint32_t* tile_val, uint32_t vmask,
                   int64_t n_keys, const float4* rec_a, const float4* rec_b, const float* rec_c,
                   int64_t n_rec, const BlendOut& o, cudaStream_t s, int bin_log2, const uint2* rec_rect,
-                  unsigned long long* pairs, uint32_t* tile_ctr) {
+                  unsigned long long* pairs, uint32_t* tile_ctr, bool chained) {
     BlendFrame f = blend_frame(cam, ranges, tile_val, vmask, n_keys, rec_a, rec_b, rec_c, n_rec, o,
                                bin_log2, rec_rect);
     if (f.ntiles == 0) return;
@@ -404,7 +405,7 @@ void launch_blend(const DevCamera& cam, const uint2* ranges, const uint32_t* til
     } else if (pairs) {
         blend_kernel<false, true><<<grid, kBlendThreads, 0, s>>>(f);
     } else {
-        blend_kernel<false, false><<<grid, kBlendThreads, 0, s>>>(f);
+        launch_chained(chained, blend_kernel<false, false>, grid, kBlendThreads, s, f);
     }
 }
 

@@ -209,9 +209,10 @@ project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict
     __shared__ uint32_t s_scan[33];
     __shared__ unsigned long long s_keys, s_bkeys;
     __shared__ uint32_t s_dh[4][256];   // depth-key digit counts (the depth sort's histogram)
-    if (threadIdx.x == 0) { s_tile = atomicAdd(tile_counter, 1u); s_keys = 0ull; s_bkeys = 0ull; }
     if (P.o.depth_hist)
         for (int j = threadIdx.x; j < 4 * 256; j += kProjThreads) (&s_dh[0][0])[j] = 0;
+    chain_wait();
+    if (threadIdx.x == 0) { s_tile = atomicAdd(tile_counter, 1u); s_keys = 0ull; s_bkeys = 0ull; }
     __syncthreads();
     const uint32_t tile = s_tile;
     const uint32_t ntiles = (uint32_t)((P.n_active + kProjThreads - 1) / kProjThreads);
@@ -480,7 +481,7 @@ cudaError_t upload_qtable(const float* q65) {
 void launch_project(const DevScene& sc, const DevCamera& cam, const uint32_t* list,
                     int64_t n_active, float tA, float tB, const ProjectOut& o, uint32_t* status,
                     uint32_t* tile_counter, uint32_t* err, cudaStream_t s,
-                    const ProjSources* src, const RawLevels* raw) {
+                    const ProjSources* src, const RawLevels* raw, bool chained) {
     ProjParams P;
     P.sc = sc;
     P.cam = cam;
@@ -499,7 +500,8 @@ void launch_project(const DevScene& sc, const DevCamera& cam, const uint32_t* li
     else if (src)
         project_kernel<kBlocks><<<(unsigned)ntiles, kProjThreads, 0, s>>>(P, status, tile_counter, err);
     else
-        project_kernel<kStore><<<(unsigned)ntiles, kProjThreads, 0, s>>>(P, status, tile_counter, err);
+        launch_chained(chained, project_kernel<kStore>, (unsigned)ntiles, kProjThreads, s, P, status, tile_counter,
+                       err);
 }
 
 size_t threshold_cost_smem(int K) { return sizeof(unsigned long long) * (2 * K + 2) + sizeof(float) * K; }

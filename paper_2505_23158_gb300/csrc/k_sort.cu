@@ -79,6 +79,7 @@ onesweep_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i < kWarps * kRadix; i += kSortThreads) (&s_whist[0][0])[i] = 0;
+    chain_wait();
     if (tid == 0) s_tile = atomicAdd(counter, 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
@@ -238,13 +239,13 @@ template <bool kWK, bool kV>
 void launch_pass(bool small, int64_t ntiles, const uint32_t* ki, const uint32_t* vi, uint32_t* ko,
                  uint32_t* vo, int64_t n, int shift, uint32_t dm, const uint32_t* off, uint32_t* st,
                  uint32_t* ctr, uint32_t* err, uint2* ranges, int range_shift, uint32_t range_tiles,
-                 const unsigned long long* d_count, bool raw, cudaStream_t s) {
+                 const unsigned long long* d_count, bool raw, cudaStream_t s, bool chained) {
     if (small)
-        onesweep_pass<kSmallIPT, kWK, kV><<<(unsigned)ntiles, kSortThreads, 0, s>>>(
-            ki, vi, ko, vo, n, shift, dm, off, st, ctr, err, ranges, range_shift, range_tiles, d_count, raw);
+        launch_chained(chained, onesweep_pass<kSmallIPT, kWK, kV>, (unsigned)ntiles, kSortThreads, s, ki, vi, ko, vo,
+                       n, shift, dm, off, st, ctr, err, ranges, range_shift, range_tiles, d_count, raw);
     else
-        onesweep_pass<kSortIPT, kWK, kV><<<(unsigned)ntiles, kSortThreads, 0, s>>>(
-            ki, vi, ko, vo, n, shift, dm, off, st, ctr, err, ranges, range_shift, range_tiles, d_count, raw);
+        launch_chained(chained, onesweep_pass<kSortIPT, kWK, kV>, (unsigned)ntiles, kSortThreads, s, ki, vi, ko, vo,
+                       n, shift, dm, off, st, ctr, err, ranges, range_shift, range_tiles, d_count, raw);
 }
 
 }  // namespace
@@ -257,7 +258,7 @@ int launch_onesweep(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t
                     int64_t n, int key_bits, void* scratch, uint32_t* err, cudaStream_t s,
                     const uint32_t* digit_offsets, bool final_keys, int shift0, uint2* ranges,
                     uint32_t range_tiles, const unsigned long long* d_count, bool scratch_cleared,
-                    bool digit_counts) {
+                    bool digit_counts, bool chained) {
     const int P = passes_for(key_bits);
     if (P == 0 || (d_count ? n < 1 : n <= 1)) return 0;
     if (d_count && !digit_offsets) return 0;   // device counts need supplied digit offsets
@@ -291,10 +292,10 @@ int launch_onesweep(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t
         const int sh = shift0 + 8 * p;
         uint2* rg = p == P - 1 ? ranges : nullptr;
         if (values) {
-            if (wk) launch_pass<true, true>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s);
-            else launch_pass<false, true>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s);
+            if (wk) launch_pass<true, true>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
+            else launch_pass<false, true>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
         } else {
-            launch_pass<true, false>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s);
+            launch_pass<true, false>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
         }
         std::swap(ki, ko);
         std::swap(vi, vo);

@@ -619,6 +619,8 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     const bool deferred = pend && !save && !importance && !sl.prof_count &&
                           sl.key_cap > 0 && na > 0 && (int)sl.pending.size() < Slot::kRing;
     if (pend) pend->used = false;
+    // (the stage profile's events would stand between the launches)
+    const bool chained = deferred && !sl.share_sms && !sl.prof_on;
     const int32_t bins_x = (cam.tiles_x + (1 << bl) - 1) >> bl;
     const int32_t bins_y = (cam.tiles_y + (1 << bl) - 1) >> bl;
     const int64_t nbins = (int64_t)bins_x * bins_y;
@@ -676,7 +678,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     prof_begin(sl, LODGE_STAGE_PROJECT, s);
     launch_project(dsc, cam, act.list, na, (float)act.tA, (float)act.tB, po,
                    ws.status.as<uint32_t>(), sl.d_small + kSmCtrProj, sl.d_small + kSmErr, s,
-                   act.blocks ? &act.src : nullptr, act.raw ? &raw : nullptr);
+                   act.blocks ? &act.src : nullptr, act.raw ? &raw : nullptr, chained);
     // (the launch count of the projection stage includes the frame's fill)
     prof_end(sl, LODGE_STAGE_PROJECT, s, (na > 0 ? 1 : 0) + (deferred ? 1 : 0));
     CUDA_TRY(cudaGetLastError());
@@ -717,7 +719,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     // (the passes scan the projection's digit counts themselves)
     int w1 = launch_onesweep(ws.dkey.as<uint32_t>(), ws.dval.as<uint32_t>(), ws.dkey2.as<uint32_t>(),
                              ws.dval2.as<uint32_t>(), n_vis, 32, ws.sort.p, sl.d_small + kSmErr, s,
-                             po.depth_hist, true, 0, nullptr, 0, d_nvis, deferred, true);
+                             po.depth_hist, true, 0, nullptr, 0, d_nvis, deferred, true, chained);
     prof_end(sl, LODGE_STAGE_DEPTH_SORT, s, onesweep_launches(n_vis, 32, true));
     DBuf& zs = w1 ? ws.dkey2 : ws.dkey;
     DBuf& rs = w1 ? ws.dval2 : ws.dval;
@@ -748,7 +750,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
         emit_n = launch_emit_counted(rs.as<uint32_t>(), n_vis, d_nvis, ws.rec_rect.as<uint2>(), bins_x, bl, n_bkeys,
                             d_nbk, ws.tkey.as<uint32_t>(), ws.tval.as<uint32_t>(), rbits, tbits,
                             ws.doffs.as<uint32_t>(), ws.status2.as<uint32_t>(), sl.d_small + kSmCtrEmit,
-                            sl.d_small + kSmErr, s);
+                            sl.d_small + kSmErr, s, chained);
     } else {
         launch_emit(rs.as<uint32_t>(), n_vis, ws.rec_rect.as<uint2>(), bins_x, bl,
                     ws.koff.as<uint32_t>(), ws.srec.as<uint32_t>(), ws.srect.as<uint2>(), n_bkeys,
@@ -775,7 +777,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
                              tbits, deferred ? ws.sort2.p : ws.sort.p, sl.d_small + kSmErr, s,
                              ws.doffs.as<uint32_t>(), true, rbits,
                              fused_ranges ? ws.ranges.as<uint2>() : nullptr, (uint32_t)nbins, d_nbk, deferred,
-                             deferred);   // deferred frames' emission leaves its digit counts unscanned
+                             deferred, chained);   // deferred frames' emission leaves its digit counts unscanned
     prof_end(sl, LODGE_STAGE_TILE_SORT, s, onesweep_launches(n_bkeys, tbits, true));
     DBuf& ks = w2 ? ws.tkey2 : ws.tkey;
     DBuf& vs = w2 ? ws.tval2 : ws.tval;
@@ -816,7 +818,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
         launch_blend(cam, ws.ranges.as<uint2>(), rec_of_pair, vmask, n_bkeys, ws.rec_a.as<float4>(),
                      ws.rec_b.as<float4>(), ws.rec_c.as<float>(), n_vis, bo, s, bl, ws.rec_rect.as<uint2>(),
                      sl.prof_count ? reinterpret_cast<unsigned long long*>(sl.d_small + kSmPairs) : nullptr,
-                     sl.share_sms ? sl.d_small + kSmCtrBlend : nullptr);
+                     sl.share_sms ? sl.d_small + kSmCtrBlend : nullptr, chained);
         if (sl.prof_count) end_sync = true;   // the counts are read back with the frame
     }
     prof_end(sl, LODGE_STAGE_BLEND, s, job ? 0 : ntiles_img > 0 ? (importance ? 1 + (n_vis > 0) : 1) : 0);
