@@ -306,24 +306,31 @@ int onesweep_launches(int64_t n, int key_bits, bool offsets_supplied);
 // per image row; a record goes to every bin its tile rect touches.  koff:
 // n_vis + 1 words; srec / srect: n_vis gathered record ids and bin rects;
 // n_keys (bin keys) from the projection's count.  digit_hist (zeroed,
-// 4 x 256 words) receives the exclusive digit offsets of the bin sort on
-// key_bits bin bits.  rbits > 0: one packed word per pair,
+// 4 x 256 words) receives the bin sort's digit counts on key_bits bin bits,
+// not scanned (launch_onesweep with digit_counts scans them).  rbits > 0: one packed word per pair,
 // bin << rbits | record (tile_val unused); rbits = 0: bin in tile_key,
-// record in tile_val.
+// record in tile_val.  Returns the launches.
 constexpr int kEmitThreads = 256;
-constexpr int kEmitKeysPerCta = 2048;   // slice of the key list (small records)
+// Tiles of depth-sorted records, one CTA each: the first kEmitNear records
+// (the nearest, which hold most of the large rects) in tiles of
+// kEmitNearTile, the others in tiles of `rest`.
+constexpr int kEmitNear = 4096;
+constexpr int kEmitNearTile = 32;
+__host__ __device__ __forceinline__ int64_t emit_tiles(int64_t n, int rest) {
+    if (n <= kEmitNear) return (n + kEmitNearTile - 1) / kEmitNearTile;
+    return kEmitNear / kEmitNearTile + (n - kEmitNear + rest - 1) / rest;
+}
 constexpr int64_t kEmitWarpMinKeys = 32;  // mean keys per record for one warp per record
-void launch_emit(const uint32_t* sorted_rec, int64_t n_vis, const uint2* rec_rect,
-                 int32_t bins_x, int bin_log2, uint32_t* koff, uint32_t* srec, uint2* srect,
-                 int64_t n_keys, uint32_t* tile_key, uint32_t* tile_val, int rbits, int key_bits,
-                 uint32_t* digit_hist, uint32_t* status, uint32_t* tile_counter, uint32_t* err,
-                 cudaStream_t s);
+int launch_emit(const uint32_t* sorted_rec, int64_t n_vis, const uint2* rec_rect,
+                int32_t bins_x, int bin_log2, uint32_t* koff, uint32_t* srec, uint2* srect,
+                int64_t n_keys, uint32_t* tile_key, uint32_t* tile_val, int rbits, int key_bits,
+                uint32_t* digit_hist, uint32_t* status, uint32_t* tile_counter, uint32_t* err,
+                cudaStream_t s);
 // The same emission with the counts on the device (one fused launch, or
 // count / scan / write above a 2^21-record capacity; bins of any size,
 // per-tile lists included): n_vis_cap and key_cap are capacities
 // (key_tile/tile_val hold key_cap words); d_nvis and d_nkeys (u64) the
-// frame's visible records and bin keys.  digit_hist receives the bin sort's
-// digit counts, not scanned (launch_onesweep with digit_counts scans them).
+// frame's visible records and bin keys (null: the capacities are the counts).
 // A frame whose keys exceed key_cap writes none and sets kErrOverflow.
 // Returns the launches.
 int launch_emit_counted(const uint32_t* sorted_rec, int64_t n_vis_cap, const unsigned long long* d_nvis,
@@ -331,10 +338,6 @@ int launch_emit_counted(const uint32_t* sorted_rec, int64_t n_vis_cap, const uns
                          const unsigned long long* d_nkeys, uint32_t* tile_key, uint32_t* tile_val,
                          int rbits, int key_bits, uint32_t* digit_hist, uint32_t* status,
                          uint32_t* tile_counter, uint32_t* err, cudaStream_t s, bool chained = false);
-
-int emit_launches(int64_t n_vis, int64_t n_keys, int bin_log2);
-// exclusive scan, in place, of `passes` 256-bin digit histograms (one launch)
-void launch_digit_scan(uint32_t* hist, int passes, cudaStream_t s);
 
 // K6: per tile [begin, end) of the sorted keys (tile = key >> shift);
 // ranges zeroed by the caller.

@@ -3,9 +3,9 @@
 // "Preliminaries: 3DGS": each 2D Gaussian is assigned to every 16x16 tile it
 // overlaps).  A bin is the tile itself or a square of 2^bin_log2 tiles; the
 // compositing then drops, per tile, the records of its bin that miss the
-// tile.  Two passes: key offsets by block scan plus decoupled look-back, then
-// emission, key-balanced for small records, one warp per record for large
-// ones.
+// tile.  Key offsets by block scan plus decoupled look-back (or count, scan and
+// write launches for large frames), the keys of a warp's records written by
+// its lanes together; frames of large records write one record per warp.
 //
 // K6: per-bin [begin, end) ranges of the bin-sorted keys.
 #include "common.cuh"
@@ -66,153 +66,109 @@ emit_offsets_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis,
     if (i < n_vis) koff[i] = s_prefix + excl;
 }
 
-// Pass 2, many small records: the key list is cut into slices of kEmitKeysPerCta keys; a CTA
-// writes whole slices (grid-stride).  The (at most kEmitKeysPerCta) records
-// that own a slice are located by one warp-parallel search in koff, staged in
-// shared memory, and each key finds its record by binary search there, so
-// every slice costs the same however large single rects are.  The CTA also
-// counts the tile sort's digits (shared-memory histograms flushed once).
-__device__ __forceinline__ int64_t warp_upper_bound(const uint32_t* __restrict__ a, int64_t n,
-                                                    uint32_t v) {
-    // last index g in [0, n) with a[g] <= v (a ascending, a[0] <= v)
-    const int lane = threadIdx.x & 31;
-    int64_t lo = 0, hi = n;
-    while (hi - lo > 32) {
-        const int64_t step = (hi - lo + 31) / 32;
-        const int64_t p = lo + (int64_t)lane * step;
-        const bool ok = p < hi && a[p] <= v;
-        const uint32_t m = __ballot_sync(0xffffffffu, ok);
-        const int last = 31 - __clz(m);   // lane 0 always qualifies
-        const int64_t nlo = lo + (int64_t)last * step;
-        hi = min(hi, nlo + step);
-        lo = nlo;
-    }
-    const int64_t p = lo + lane;
-    const bool ok = p < hi && a[p] <= v;
-    const uint32_t m = __ballot_sync(0xffffffffu, ok);
-    return lo + (31 - __clz(m));
-}
+// What a CTA needs to write its records' keys.
+struct KeyWriter {
+    int32_t bins_x;
+    uint32_t* tile_key;
+    uint32_t* tile_val;
+    int rbits, passes;
+    uint32_t last_mask;
+    uint32_t (*hist)[256];   // the bin sort's digit counts, shared memory
 
-__global__ void __launch_bounds__(kEmitThreads)
-emit_keys_sliced_kernel(const uint32_t* __restrict__ koff, const uint32_t* __restrict__ srec,
-                 const uint2* __restrict__ srect, int64_t n_vis, int64_t n_keys, int32_t tiles_x,
-                 uint32_t* __restrict__ tile_key, uint32_t* __restrict__ tile_val, int rbits,
-                 int passes, uint32_t last_mask, uint32_t* __restrict__ digit_hist,
-                 uint32_t* __restrict__ err) {
-    __shared__ uint32_t s_off[kEmitKeysPerCta + 1];
-    __shared__ uint2 s_rect[kEmitKeysPerCta];
-    __shared__ uint32_t s_rec[kEmitKeysPerCta];
-    __shared__ uint32_t s_hist[3][256];
-    __shared__ int64_t s_g0;
-    __shared__ int s_m;
-    for (int i = threadIdx.x; i < 3 * 256; i += kEmitThreads) (&s_hist[0][0])[i] = 0;
-    const int64_t nslices = (n_keys + kEmitKeysPerCta - 1) / kEmitKeysPerCta;
-    for (int64_t sl = blockIdx.x; sl < nslices; sl += gridDim.x) {
-        const int64_t k0 = sl * kEmitKeysPerCta;
-        const int64_t k1 = min(k0 + (int64_t)kEmitKeysPerCta, n_keys);
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            const int64_t g0 = warp_upper_bound(koff, n_vis, (uint32_t)k0);
-            const int64_t g1 = warp_upper_bound(koff + g0, n_vis - g0, (uint32_t)(k1 - 1)) + g0;
-            if (threadIdx.x == 0) {
-                int64_t m = g1 - g0 + 1;
-                if (m > kEmitKeysPerCta) { atomicOr(err, kErrOverflow); m = kEmitKeysPerCta; }
-                s_g0 = g0;
-                s_m = (int)m;
-            }
+    __device__ __forceinline__ void put(int64_t at, uint32_t bin, uint32_t rec) const {
+        if (rbits) {
+            tile_key[at] = (bin << rbits) | rec;
+        } else {
+            tile_key[at] = bin;
+            tile_val[at] = rec;
         }
-        __syncthreads();
-        const int64_t g0 = s_g0;
-        const int m = s_m;
-        for (int j = threadIdx.x; j < m; j += kEmitThreads) {
-            s_off[j] = koff[g0 + j];
-            s_rect[j] = srect[g0 + j];
-            s_rec[j] = srec[g0 + j];
-        }
-        __syncthreads();
-        for (int64_t key = k0 + threadIdx.x; key < k1; key += kEmitThreads) {
-            int lo = 0, hi = m;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (s_off[mid] <= (uint32_t)key) lo = mid; else hi = mid;
+        atomicAdd(&hist[0][bin & (passes == 1 ? last_mask : 0xffu)], 1u);
+    }
+    // the digits above the lowest, counted per row of a record's bins
+    // [x0, x0 + w): one contiguous range of ids, split where a digit changes
+    __device__ __forceinline__ void count_row(uint32_t x0, uint32_t y, uint32_t w) const {
+        for (int p = 1; p < passes; ++p) {
+            const uint32_t mask = p == passes - 1 ? last_mask : 0xffu;
+            const int sh = 8 * p;
+            uint32_t a = y * (uint32_t)bins_x + x0;
+            const uint32_t b = a + w - 1u;
+            while (a <= b) {
+                const uint32_t end = min(b, ((a >> sh) + 1u << sh) - 1u);
+                atomicAdd(&hist[p][(a >> sh) & mask], end - a + 1u);
+                a = end + 1u;
             }
-            const uint32_t k = (uint32_t)key - s_off[lo];
-            const uint2 rr = s_rect[lo];
-            const uint32_t tx0 = rr.x & 0xffffu, ty0 = rr.x >> 16, tx1 = rr.y & 0xffffu;
-            const uint32_t w = tx1 - tx0 + 1u;
-            const uint32_t q = k / w;
-            const uint32_t tile = (ty0 + q) * (uint32_t)tiles_x + tx0 + (k - q * w);
-            if (rbits) {
-                tile_key[key] = (tile << rbits) | s_rec[lo];
-            } else {
-                tile_key[key] = tile;
-                tile_val[key] = s_rec[lo];
-            }
-            for (int p = 0; p < passes; ++p)
-                atomicAdd(&s_hist[p][(tile >> (8 * p)) & (p == passes - 1 ? last_mask : 0xffu)], 1u);
         }
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < passes * 256; i += kEmitThreads) {
-        const uint32_t c = (&s_hist[0][0])[i];
-        if (c) atomicAdd(digit_hist + i, c);
+    // The keys of a warp's records, one record per lane: cnt keys (w bins a
+    // row from (x0, y0)) at position `at`; lanes with nothing to write have
+    // cnt = 0.  The lanes take consecutive keys: a key's record is found by
+    // a binary search over the lanes' running counts, so that a warp takes
+    // as many turns as it has keys / 32 and stores whole sectors, instead of
+    // as many as its largest record has keys, each lane storing its own run.
+    __device__ __forceinline__ void warp_records(uint32_t cnt, uint32_t at, uint32_t x0, uint32_t y0, uint32_t w,
+                                                 uint32_t rec) const {
+        const int lane = threadIdx.x & 31;
+        uint32_t incl = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const uint32_t excl = incl - cnt, total = __shfl_sync(0xffffffffu, incl, 31);
+        const uint32_t xy = x0 | (y0 << 16);   // bin coordinates < 2^16
+        for (uint32_t k0 = 0; k0 < total; k0 += 32) {
+            const uint32_t k = k0 + lane;
+            int own = 0;   // the last lane with excl <= k
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(0xffffffffu, excl, own + step) <= k) own += step;
+            const uint32_t j = k - __shfl_sync(0xffffffffu, excl, own);
+            const uint32_t oxy = __shfl_sync(0xffffffffu, xy, own), ow = __shfl_sync(0xffffffffu, w, own);
+            const uint32_t oat = __shfl_sync(0xffffffffu, at, own), orec = __shfl_sync(0xffffffffu, rec, own);
+            if (k < total) {
+                // j, w <= kWarpKeys: j + 1/2 is 1/(2 w) of a row or more from
+                // a whole one, far above the quotient's error
+                const uint32_t row = (uint32_t)__fdividef((float)j + 0.5f, (float)ow);
+                put((int64_t)oat + j, ((oxy >> 16) + row) * (uint32_t)bins_x + (oxy & 0xffffu) + (j - row * ow), orec);
+            }
+        }
+        if (cnt)
+            for (uint32_t r = 0; r * w < cnt; ++r) count_row(x0, y0 + r, w);
     }
-}
+    // one record by a whole warp
+    __device__ __forceinline__ void large_record(uint32_t cnt, int64_t at, uint32_t x0, uint32_t y0, uint32_t w,
+                                                 uint32_t rec) const {
+        const int lane = threadIdx.x & 31;
+        // key k = lane + 32 j sits at row k / w, column k % w (stepped)
+        uint32_t row = lane / w, col = lane - row * w;
+        const uint32_t drow = 32u / w, dcol = 32u - drow * w;
+        for (uint32_t k = lane; k < cnt; k += 32) {
+            put(at + k, (y0 + row) * (uint32_t)bins_x + x0 + col, rec);
+            row += drow;
+            col += dcol;
+            if (col >= w) { col -= w; ++row; }
+        }
+        for (uint32_t r = lane; r * w < cnt; r += 32) count_row(x0, y0 + r, w);
+    }
+};
 
-// Pass 2, large records: one warp per depth-sorted record writes the record's keys,
-// koff[i] .. koff[i+1]-1, its rect row-major, the lanes striding over them
-// (warps of a CTA take consecutive records, CTAs stride over the list).  The
-// CTA also counts the tile sort's digits in shared-memory histograms flushed
-// once: the lowest digit per key (consecutive tiles fall in different bins),
-// the higher digits per rect row, whose tile ids are one contiguous range
-// that crosses a digit boundary at most once per 256 tiles.
+// Large records: one warp per depth-sorted record writes the record's keys,
+// koff[i] .. koff[i+1]-1 (warps of a CTA take consecutive records, CTAs
+// stride over the list).
 __global__ void __launch_bounds__(kEmitThreads)
 emit_keys_rect_kernel(const uint32_t* __restrict__ koff, const uint32_t* __restrict__ srec,
-                 const uint2* __restrict__ srect, int64_t n_vis, int32_t tiles_x,
+                 const uint2* __restrict__ srect, int64_t n_vis, int32_t bins_x,
                  uint32_t* __restrict__ tile_key, uint32_t* __restrict__ tile_val, int rbits,
                  int passes, uint32_t last_mask, uint32_t* __restrict__ digit_hist) {
     __shared__ uint32_t s_hist[3][256];
     for (int i = threadIdx.x; i < 3 * 256; i += kEmitThreads) (&s_hist[0][0])[i] = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31;
+    const KeyWriter kw{bins_x, tile_key, tile_val, rbits, passes, last_mask, s_hist};
     const int64_t wstride = (int64_t)gridDim.x * (kEmitThreads / 32);
     for (int64_t i = (int64_t)blockIdx.x * (kEmitThreads / 32) + (threadIdx.x >> 5); i < n_vis;
          i += wstride) {
-        const uint32_t k0 = koff[i];
-        const uint32_t cnt = koff[i + 1] - k0;
         const uint2 rr = srect[i];
-        const uint32_t rec = srec[i];
-        const uint32_t tx0 = rr.x & 0xffffu, ty0 = rr.x >> 16;
-        const uint32_t w = (rr.y & 0xffffu) - tx0 + 1u, h = (rr.y >> 16) - ty0 + 1u;
-        // key k = lane + 32 j sits at row k / w, column k % w (stepped)
-        uint32_t row = lane / w, col = lane - row * w;
-        const uint32_t drow = 32u / w, dcol = 32u - drow * w;
-        for (uint32_t k = lane; k < cnt; k += 32) {
-            const uint32_t tile = (ty0 + row) * (uint32_t)tiles_x + tx0 + col;
-            if (rbits) {
-                tile_key[k0 + k] = (tile << rbits) | rec;
-            } else {
-                tile_key[k0 + k] = tile;
-                tile_val[k0 + k] = rec;
-            }
-            atomicAdd(&s_hist[0][tile & (passes == 1 ? last_mask : 0xffu)], 1u);
-            row += drow;
-            col += dcol;
-            if (col >= w) { col -= w; ++row; }
-        }
-        for (int p = 1; p < passes; ++p) {
-            const uint32_t mask = p == passes - 1 ? last_mask : 0xffu;
-            const int sh = 8 * p;
-            for (uint32_t r = lane; r < h; r += 32) {
-                uint32_t a = (ty0 + r) * (uint32_t)tiles_x + tx0;
-                const uint32_t b = a + w - 1u;
-                while (a <= b) {   // split [a, b] where digit p changes
-                    const uint32_t end = min(b, ((a >> sh) + 1u << sh) - 1u);
-                    atomicAdd(&s_hist[p][(a >> sh) & mask], end - a + 1u);
-                    a = end + 1u;
-                }
-            }
-        }
+        kw.large_record(koff[i + 1] - koff[i], koff[i], rr.x & 0xffffu, rr.x >> 16,
+                        (rr.y & 0xffffu) - (rr.x & 0xffffu) + 1u, srec[i]);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < passes * 256; i += kEmitThreads) {
@@ -221,14 +177,27 @@ emit_keys_rect_kernel(const uint32_t* __restrict__ koff, const uint32_t* __restr
     }
 }
 
-// Coarse bins (a few keys per record): offsets and emission in one pass.
-// A CTA takes 256 depth-sorted records, scans their bin counts and finds
-// its key offset by decoupled look-back.  A record of at most 32 keys is
-// written by its own thread; larger ones (the nearest records, which all
-// fall in the first CTAs) go to a shared list that the CTA's warps take one
-// record at a time, the lanes striding over the record's keys.  The bin
-// sort's digit counts are kept in shared memory and flushed once.
-constexpr uint32_t kFusedThreadKeys = 32;
+// Tile t of depth-sorted records: the first one, and how many (before the
+// end of the list is taken into account).  With equal tiles the CTAs of the
+// nearest records wrote most of the keys while the others had finished: four
+// full-detail 1080p frames 1908 -> 1771 us, an LOD frame 286 -> 271 us (with
+// the first 1024 records instead of 4096 in near tiles 1825 and 265).
+__device__ __forceinline__ int64_t emit_first(uint32_t t, int rest, int& size) {
+    constexpr uint32_t kNearTiles = kEmitNear / kEmitNearTile;
+    size = t < kNearTiles ? kEmitNearTile : rest;
+    return t < kNearTiles ? (int64_t)t * kEmitNearTile : kEmitNear + (int64_t)(t - kNearTiles) * rest;
+}
+
+// Offsets and emission in one pass.  A CTA takes a tile of depth-sorted records,
+// scans their bin counts and finds its key offset by decoupled look-back.
+// Records of at most kWarpKeys keys are written by their warp together; larger
+// ones (the nearest records, which all fall in the first CTAs) go to a shared
+// list that the CTA's warps take one record at a time.  The bin sort's digit
+// counts are kept in shared memory and flushed once.  Bound by the latency of
+// its chain (ticket, records, look-back), not by its bytes: a chunk frame's
+// 124k records and 450k keys take 16.5 us where a thread writing its own
+// record's keys took 25.8.
+constexpr uint32_t kWarpKeys = 32;   // at most 2^10 (warp_records)
 __global__ void __launch_bounds__(kEmitThreads)
 emit_fused_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis,
                   const uint2* __restrict__ rec_rect, int bin_log2, int32_t bins_x, int64_t n_keys,
@@ -258,11 +227,12 @@ emit_fused_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis,
     if (threadIdx.x == 0) { s_tile = atomicAdd(counter, 1u); s_nbig = 0; }
     __syncthreads();
     const uint32_t tile = s_tile;
-    const uint32_t ntiles = (uint32_t)((n_vis + kEmitThreads - 1) / kEmitThreads);
+    const uint32_t ntiles = (uint32_t)emit_tiles(n_vis, kEmitThreads);
     if (tile >= ntiles) return;   // past the device count (later tiles too)
-    const int64_t i = (int64_t)tile * kEmitThreads + threadIdx.x;
+    int size;
+    const int64_t i = emit_first(tile, kEmitThreads, size) + threadIdx.x;
     uint32_t cnt = 0, rec = 0, x0 = 0, y0 = 0, w = 1;
-    if (i < n_vis) {
+    if ((int)threadIdx.x < size && i < n_vis) {
         rec = sorted_rec[i];
         if ((int64_t)rec >= n_vis) { atomicOr(err, kErrBadIndex); rec = 0; }
         const uint2 p = rec_rect[rec];   // pixel range -> tile range -> bin range
@@ -274,7 +244,7 @@ emit_fused_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis,
     }
     uint32_t total;
     const uint32_t excl = block_exclusive_scan(cnt, s_scan, &total);
-    if (cnt > kFusedThreadKeys) {
+    if (cnt > kWarpKeys) {
         const uint32_t slot = atomicAdd(&s_nbig, 1u);
         s_big[slot] = threadIdx.x;
         s_off[threadIdx.x] = excl;
@@ -303,48 +273,13 @@ emit_fused_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis,
         if (threadIdx.x == 0) atomicOr(err, kErrOverflow);
         return;
     }
-    // small records: the owning thread
-    if (cnt <= kFusedThreadKeys) {
-        uint32_t row = 0, col = 0;
-        for (uint32_t k = 0; k < cnt; ++k) {
-            const uint32_t bin = (y0 + row) * (uint32_t)bins_x + x0 + col;
-            const int64_t at = base + excl + k;
-            if (rbits) {
-                tile_key[at] = (bin << rbits) | rec;
-            } else {
-                tile_key[at] = bin;
-                tile_val[at] = rec;
-            }
-            for (int p = 0; p < passes; ++p)
-                atomicAdd(&s_hist[p][(bin >> (8 * p)) & (p == passes - 1 ? last_mask : 0xffu)], 1u);
-            if (++col == w) { col = 0; ++row; }
-        }
-    }
-    // large records: one warp each
-    const int lane = threadIdx.x & 31;
+    const KeyWriter kw{bins_x, tile_key, tile_val, rbits, passes, last_mask, s_hist};
+    kw.warp_records(cnt <= kWarpKeys ? cnt : 0u, (uint32_t)base + excl, x0, y0, w, rec);
     const uint32_t nbig = s_nbig;
     for (uint32_t b = threadIdx.x >> 5; b < nbig; b += kEmitThreads / 32) {
         const uint32_t t = s_big[b];
         const uint2 rr = s_rect[t];
-        const uint32_t bx0 = rr.x & 0xffffu, by0 = rr.x >> 16, bw = rr.y, bc = s_cnt[t];
-        const uint32_t brec = s_rec[t];
-        const int64_t at0 = base + s_off[t];
-        uint32_t row = lane / bw, col = lane - row * bw;
-        const uint32_t drow = 32u / bw, dcol = 32u - drow * bw;
-        for (uint32_t k = lane; k < bc; k += 32) {
-            const uint32_t bin = (by0 + row) * (uint32_t)bins_x + bx0 + col;
-            if (rbits) {
-                tile_key[at0 + k] = (bin << rbits) | brec;
-            } else {
-                tile_key[at0 + k] = bin;
-                tile_val[at0 + k] = brec;
-            }
-            for (int p = 0; p < passes; ++p)
-                atomicAdd(&s_hist[p][(bin >> (8 * p)) & (p == passes - 1 ? last_mask : 0xffu)], 1u);
-            row += drow;
-            col += dcol;
-            if (col >= bw) { col -= bw; ++row; }
-        }
+        kw.large_record(s_cnt[t], base + s_off[t], rr.x & 0xffffu, rr.x >> 16, rr.y, s_rec[t]);
     }
     __syncthreads();
     for (int j = threadIdx.x; j < passes * 256; j += kEmitThreads) {
@@ -386,13 +321,15 @@ emit_count_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
     __shared__ uint32_t s_part[kEmitThreads / 32];
     chain_wait();
     const int64_t n_vis = device_count(n_vis_cap, d_nvis);
-    const int64_t t0 = (int64_t)blockIdx.x * kEmitTileRecs;
+    int size;
+    const int64_t t0 = emit_first(blockIdx.x, kEmitTileRecs, size);
     if (t0 >= n_vis) return;   // past the device count (later tiles too)
+    const int64_t t1 = min(n_vis, t0 + size);
     uint32_t sum = 0;
 #pragma unroll
     for (int j = 0; j < kEmitRecs; ++j) {
         const int64_t i = t0 + (int64_t)j * kEmitThreads + threadIdx.x;
-        if (i < n_vis) {
+        if (i < t1) {
             uint32_t rec = sorted_rec[i];
             if ((int64_t)rec >= n_vis) { atomicOr(err, kErrBadIndex); rec = 0; }
             uint32_t x0, y0, w;
@@ -417,7 +354,7 @@ emit_scan_kernel(int tile_recs, uint32_t* __restrict__ tile_sum, int64_t n_vis_c
     __shared__ uint32_t s_scan[33];
     chain_wait();
     const int64_t n_vis = device_count(n_vis_cap, d_nvis);
-    const int64_t ntiles = (n_vis + tile_recs - 1) / tile_recs;
+    const int64_t ntiles = emit_tiles(n_vis, tile_recs);
     uint64_t carry = 0;
     for (int64_t base = 0; base < ntiles; base += 1024) {
         const int64_t t = base + threadIdx.x;
@@ -448,8 +385,10 @@ emit_write_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
     __shared__ uint32_t s_hist[3][256];
     chain_wait();
     const int64_t n_vis = device_count(n_vis_cap, d_nvis);
-    const int64_t t0 = (int64_t)blockIdx.x * kEmitTileRecs;
+    int size;
+    const int64_t t0 = emit_first(blockIdx.x, kEmitTileRecs, size);
     if (t0 >= n_vis) return;
+    const int64_t t1 = min(n_vis, t0 + size);
     for (int i = threadIdx.x; i < 3 * 256; i += kEmitThreads) (&s_hist[0][0])[i] = 0;
     if (threadIdx.x == 0) s_nbig = 0;
     // a thread's records are j * kEmitThreads + thread, so that the loads
@@ -460,13 +399,14 @@ emit_write_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
     for (int j = 0; j < kEmitRecs; ++j) {
         const int64_t i = t0 + (int64_t)j * kEmitThreads + threadIdx.x;
         rec[j] = 0; cnt[j] = 0; bx[j] = 0; by[j] = 0; bw[j] = 1;
-        if (i < n_vis) {
+        if (i < t1) {
             rec[j] = sorted_rec[i];
             if ((int64_t)rec[j] >= n_vis) rec[j] = 0;   // flagged by the count kernel
             cnt[j] = rec_bin_rect(rec_rect, rec[j], bin_log2, bx[j], by[j], bw[j]);
         }
     }
     const int64_t tbase = tile_off[blockIdx.x];
+    const KeyWriter kw{bins_x, tile_key, tile_val, rbits, passes, last_mask, s_hist};
     uint32_t run = 0;   // keys of the record groups before group j in this tile
     __syncthreads();   // s_hist and s_nbig are set
 #pragma unroll
@@ -474,34 +414,22 @@ emit_write_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
         uint32_t total;
         const uint32_t excl = block_exclusive_scan(cnt[j], s_scan, &total);
         const int64_t at0 = tbase + run + excl;
+        uint32_t mine = cnt[j];
         if (at0 + cnt[j] > key_cap) {
             if (cnt[j]) atomicOr(err, kErrOverflow);
-        } else if (cnt[j] > kFusedThreadKeys) {
+            mine = 0;
+        } else if (cnt[j] > kWarpKeys) {
             const uint32_t slot = atomicAdd(&s_nbig, 1u);
             s_big[slot] = (threadIdx.x << 2) | (uint32_t)j;
             s_off[slot] = run + excl;
-        } else {
-            uint32_t row = 0, col = 0;
-            for (uint32_t k = 0; k < cnt[j]; ++k) {
-                const uint32_t bin = (by[j] + row) * (uint32_t)bins_x + bx[j] + col;
-                const int64_t at = at0 + k;
-                if (rbits) {
-                    tile_key[at] = (bin << rbits) | rec[j];
-                } else {
-                    tile_key[at] = bin;
-                    tile_val[at] = rec[j];
-                }
-                for (int p = 0; p < passes; ++p)
-                    atomicAdd(&s_hist[p][(bin >> (8 * p)) & (p == passes - 1 ? last_mask : 0xffu)], 1u);
-                if (++col == bw[j]) { col = 0; ++row; }
-            }
+            mine = 0;
         }
+        kw.warp_records(mine, (uint32_t)at0, bx[j], by[j], bw[j], rec[j]);
         // the next record group's keys follow this group's
         run += total;
     }
     __syncthreads();
     // records with many keys: one warp each; their rects are read again
-    const int lane = threadIdx.x & 31;
     const uint32_t nbig = s_nbig;
     for (uint32_t b = threadIdx.x >> 5; b < nbig; b += kEmitThreads / 32) {
         const uint32_t tj = s_big[b];
@@ -510,37 +438,13 @@ emit_write_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
         if ((int64_t)r >= n_vis) r = 0;
         uint32_t x0, y0, w;
         const uint32_t c = rec_bin_rect(rec_rect, r, bin_log2, x0, y0, w);
-        const int64_t at0 = tbase + s_off[b];
-        uint32_t row = lane / w, col = lane - row * w;
-        const uint32_t drow = 32u / w, dcol = 32u - drow * w;
-        for (uint32_t k = lane; k < c; k += 32) {
-            const uint32_t bin = (y0 + row) * (uint32_t)bins_x + x0 + col;
-            if (rbits) {
-                tile_key[at0 + k] = (bin << rbits) | r;
-            } else {
-                tile_key[at0 + k] = bin;
-                tile_val[at0 + k] = r;
-            }
-            for (int p = 0; p < passes; ++p)
-                atomicAdd(&s_hist[p][(bin >> (8 * p)) & (p == passes - 1 ? last_mask : 0xffu)], 1u);
-            row += drow;
-            col += dcol;
-            if (col >= w) { col -= w; ++row; }
-        }
+        kw.large_record(c, tbase + s_off[b], x0, y0, w, r);
     }
     __syncthreads();
     for (int j = threadIdx.x; j < passes * 256; j += kEmitThreads) {
         const uint32_t c = (&s_hist[0][0])[j];
         if (c) atomicAdd(digit_hist + j, c);
     }
-}
-
-// exclusive scan of each pass's 256-bin digit histogram, in place
-__global__ void digit_scan_kernel(uint32_t* hist) {
-    __shared__ uint32_t s_scan[33];
-    uint32_t* h = hist + blockIdx.x * 256;
-    uint32_t v = h[threadIdx.x], total;
-    h[threadIdx.x] = block_exclusive_scan(v, s_scan, &total);
 }
 
 // K6: per tile [begin, end) of the tile-sorted keys (tile = key >> shift);
@@ -566,43 +470,34 @@ __global__ void ranges_kernel(const uint32_t* __restrict__ key, int64_t n, uint2
 
 }  // namespace
 
-void launch_emit(const uint32_t* sorted_rec, int64_t n_vis, const uint2* rec_rect,
-                 int32_t bins_x, int bin_log2, uint32_t* koff, uint32_t* srec, uint2* srect,
-                 int64_t n_keys, uint32_t* tile_key, uint32_t* tile_val, int rbits, int key_bits,
-                 uint32_t* digit_hist, uint32_t* status, uint32_t* tile_counter, uint32_t* err,
-                 cudaStream_t s) {
-    const int32_t tiles_x = bins_x;   // the emit kernels index bins as tiles
-    int64_t nb = (n_vis + kEmitThreads - 1) / kEmitThreads;
-    if (nb == 0) return;
+// digits of the bin ids: passes and the mask of the last one
+static void bin_digits(int key_bits, int* passes, uint32_t* last_mask) {
     const int P = (key_bits + 7) / 8;
     const int last_bits = key_bits - 8 * (P - 1);
-    const uint32_t last_mask = last_bits >= 8 ? 0xffu : ((1u << last_bits) - 1u);
-    if (n_keys > 0 && n_keys < kEmitWarpMinKeys * n_vis && bin_log2 > 0) {
-        // coarse bins: a few keys per record, one fused pass
-        emit_fused_kernel<<<(unsigned)nb, kEmitThreads, 0, s>>>(sorted_rec, n_vis, rec_rect, bin_log2, bins_x,
-                                                                n_keys, tile_key, tile_val, rbits, P, last_mask,
-                                                                digit_hist, status, tile_counter, err, nullptr,
-                                                                nullptr);
-        digit_scan_kernel<<<P, 256, 0, s>>>(digit_hist);
-        return;
-    }
-    emit_offsets_kernel<<<(unsigned)nb, kEmitThreads, 0, s>>>(sorted_rec, n_vis, rec_rect, koff, srec,
-                                                              srect, bin_log2, status, tile_counter, err);
-    if (n_keys == 0) return;
-    if (n_keys >= kEmitWarpMinKeys * n_vis) {
-        // records average a warp's worth of keys or more: one warp per record
-        const unsigned grid = (unsigned)std::min<int64_t>((n_vis + kEmitThreads / 32 - 1) / (kEmitThreads / 32),
-                                                          (int64_t)device_sms() * 8);
-        emit_keys_rect_kernel<<<grid, kEmitThreads, 0, s>>>(koff, srec, srect, n_vis, tiles_x, tile_key,
-                                                            tile_val, rbits, P, last_mask, digit_hist);
-    } else {
-        const int64_t nslices = (n_keys + kEmitKeysPerCta - 1) / kEmitKeysPerCta;
-        const unsigned grid = (unsigned)std::min<int64_t>(nslices, (int64_t)device_sms() * 4);
-        emit_keys_sliced_kernel<<<grid, kEmitThreads, 0, s>>>(koff, srec, srect, n_vis, n_keys, tiles_x,
-                                                              tile_key, tile_val, rbits, P, last_mask,
-                                                              digit_hist, err);
-    }
-    digit_scan_kernel<<<P, 256, 0, s>>>(digit_hist);
+    *passes = P;
+    *last_mask = last_bits >= 8 ? 0xffu : ((1u << last_bits) - 1u);
+}
+
+int launch_emit(const uint32_t* sorted_rec, int64_t n_vis, const uint2* rec_rect,
+                int32_t bins_x, int bin_log2, uint32_t* koff, uint32_t* srec, uint2* srect,
+                int64_t n_keys, uint32_t* tile_key, uint32_t* tile_val, int rbits, int key_bits,
+                uint32_t* digit_hist, uint32_t* status, uint32_t* tile_counter, uint32_t* err,
+                cudaStream_t s) {
+    if (n_vis == 0 || n_keys == 0) return 0;
+    if (n_keys < kEmitWarpMinKeys * n_vis)
+        return launch_emit_counted(sorted_rec, n_vis, nullptr, rec_rect, bins_x, bin_log2, n_keys, nullptr,
+                                   tile_key, tile_val, rbits, key_bits, digit_hist, status, tile_counter, err, s);
+    // records average a warp's worth of keys or more: one warp per record
+    int P;
+    uint32_t last_mask;
+    bin_digits(key_bits, &P, &last_mask);
+    emit_offsets_kernel<<<(unsigned)((n_vis + kEmitThreads - 1) / kEmitThreads), kEmitThreads, 0, s>>>(
+        sorted_rec, n_vis, rec_rect, koff, srec, srect, bin_log2, status, tile_counter, err);
+    const unsigned grid = (unsigned)std::min<int64_t>((n_vis + kEmitThreads / 32 - 1) / (kEmitThreads / 32),
+                                                      (int64_t)device_sms() * 8);
+    emit_keys_rect_kernel<<<grid, kEmitThreads, 0, s>>>(koff, srec, srect, n_vis, bins_x, tile_key,
+                                                        tile_val, rbits, P, last_mask, digit_hist);
+    return 2;
 }
 
 int launch_emit_counted(const uint32_t* sorted_rec, int64_t n_vis_cap, const unsigned long long* d_nvis,
@@ -610,15 +505,15 @@ int launch_emit_counted(const uint32_t* sorted_rec, int64_t n_vis_cap, const uns
                         const unsigned long long* d_nkeys, uint32_t* tile_key, uint32_t* tile_val,
                         int rbits, int key_bits, uint32_t* digit_hist, uint32_t* status,
                         uint32_t* tile_counter, uint32_t* err, cudaStream_t s, bool chained) {
-    const int64_t nb = (n_vis_cap + kEmitThreads - 1) / kEmitThreads;
+    const int64_t nb = emit_tiles(n_vis_cap, kEmitThreads);
     if (nb == 0) return 0;
-    const int P = (key_bits + 7) / 8;
-    const int last_bits = key_bits - 8 * (P - 1);
-    const uint32_t last_mask = last_bits >= 8 ? 0xffu : ((1u << last_bits) - 1u);
+    int P;
+    uint32_t last_mask;
+    bin_digits(key_bits, &P, &last_mask);
     if (n_vis_cap > kEmitSplitMin) {
         // count, scan, write (the tile counts and offsets live in `status`,
-        // which holds one word per 256 records)
-        const unsigned nt = (unsigned)((n_vis_cap + 4 * kEmitThreads - 1) / (4 * kEmitThreads));
+        // which holds a word per tile of the fused kernel)
+        const unsigned nt = (unsigned)emit_tiles(n_vis_cap, 4 * kEmitThreads);
         launch_chained(chained, emit_count_kernel<4>, nt, kEmitThreads, s, sorted_rec, n_vis_cap, d_nvis, rec_rect, bin_log2,
                                                          status, err);
         launch_chained(chained, emit_scan_kernel, 1, 1024, s, 4 * kEmitThreads, status, n_vis_cap, d_nvis, key_cap, d_nkeys, err);
@@ -632,16 +527,6 @@ int launch_emit_counted(const uint32_t* sorted_rec, int64_t n_vis_cap, const uns
                                                             digit_hist, status, tile_counter, err, d_nvis,
                                                             d_nkeys);
     return 1;
-}
-
-void launch_digit_scan(uint32_t* hist, int passes, cudaStream_t s) {
-    if (passes > 0) digit_scan_kernel<<<passes, 256, 0, s>>>(hist);
-}
-
-int emit_launches(int64_t n_vis, int64_t n_keys, int bin_log2) {
-    if (n_vis == 0) return 0;
-    if (n_keys > 0 && n_keys < kEmitWarpMinKeys * n_vis && bin_log2 > 0) return 2;
-    return n_keys > 0 ? 3 : 1;
 }
 
 void launch_ranges(const uint32_t* tile_key, int64_t n_keys, uint2* ranges, int64_t ntiles,

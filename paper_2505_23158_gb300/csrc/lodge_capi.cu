@@ -630,7 +630,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
         // set by one launch: look-back words of the projection and the
         // emission, the slot's small words, both digit histograms, both sorts'
         // counters and look-back words, the bin ranges (begin ~0, end 0)
-        const int64_t etiles = std::max<int64_t>((na + kEmitThreads - 1) / kEmitThreads, 1);
+        const int64_t etiles = std::max<int64_t>(emit_tiles(na, kEmitThreads), 1);
         TRY(ensure(ctx, ws.status2, sizeof(uint32_t) * (size_t)etiles, s));
         TRY(ensure(ctx, ws.sort, sort_scratch_bytes(na, 32), s));
         TRY(ensure(ctx, ws.sort2, sort_scratch_bytes(sl.key_cap, tbits), s));
@@ -740,7 +740,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     TRY(ensure(ctx, ws.srec, sizeof(uint32_t) * nv1, s));
     TRY(ensure(ctx, ws.srect, sizeof(uint2) * nv1, s));
     if (!deferred) {
-        int64_t etiles = std::max<int64_t>((n_vis + kEmitThreads - 1) / kEmitThreads, 1);
+        const int64_t etiles = std::max<int64_t>(emit_tiles(n_vis, kEmitThreads), 1);
         TRY(ensure(ctx, ws.status, sizeof(uint32_t) * (size_t)etiles, s));
         CUDA_TRY(cudaMemsetAsync(ws.status.p, 0, sizeof(uint32_t) * (size_t)etiles, s));
     }
@@ -752,12 +752,12 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
                             ws.doffs.as<uint32_t>(), ws.status2.as<uint32_t>(), sl.d_small + kSmCtrEmit,
                             sl.d_small + kSmErr, s, chained);
     } else {
-        launch_emit(rs.as<uint32_t>(), n_vis, ws.rec_rect.as<uint2>(), bins_x, bl,
+        emit_n = launch_emit(rs.as<uint32_t>(), n_vis, ws.rec_rect.as<uint2>(), bins_x, bl,
                     ws.koff.as<uint32_t>(), ws.srec.as<uint32_t>(), ws.srect.as<uint2>(), n_bkeys,
                     ws.tkey.as<uint32_t>(), ws.tval.as<uint32_t>(), rbits, tbits, ws.doffs.as<uint32_t>(),
                     ws.status.as<uint32_t>(), sl.d_small + kSmCtrEmit, sl.d_small + kSmErr, s);
     }
-    prof_end(sl, LODGE_STAGE_EMIT, s, deferred ? emit_n : emit_launches(n_vis, n_bkeys, bl));
+    prof_end(sl, LODGE_STAGE_EMIT, s, emit_n);
 
     // ---- K6 bin ranges: recorded by the bin sort's last pass (begin by
     // atomic minimum from 0xffffffff, end by atomic maximum from 0); with at
@@ -777,7 +777,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
                              tbits, deferred ? ws.sort2.p : ws.sort.p, sl.d_small + kSmErr, s,
                              ws.doffs.as<uint32_t>(), true, rbits,
                              fused_ranges ? ws.ranges.as<uint2>() : nullptr, (uint32_t)nbins, d_nbk, deferred,
-                             deferred, chained);   // deferred frames' emission leaves its digit counts unscanned
+                             true, chained);   // (the emission leaves its digit counts unscanned)
     prof_end(sl, LODGE_STAGE_TILE_SORT, s, onesweep_launches(n_bkeys, tbits, true));
     DBuf& ks = w2 ? ws.tkey2 : ws.tkey;
     DBuf& vs = w2 ? ws.tval2 : ws.tval;
