@@ -427,12 +427,15 @@ void launch_blend_batch(const BlendFrame* frames, int n, cudaStream_t s, uint32_
 // K12: importance score: the blend's walk, and per record the largest
 // weight T * alpha it receives (rec_score, n_rec words, zeroed, FP32 bits),
 // then score[gid] (n_total floats, non-negative) raised to it.  rgb as in
-// launch_blend.
+// launch_blend, tile_ctr too.  d_nvis: null, or the visible count on the
+// device (n_rec is then a capacity).  err: a frame whose keys outgrew their
+// capacity (kErrOverflow) raises no score; it is rendered again.
 void launch_importance(const DevCamera& cam, const uint2* ranges, const uint32_t* tile_val,
                        uint32_t vmask, int64_t n_keys, const float4* rec_a, const float4* rec_b,
                        const float* rec_c, int64_t n_rec, const uint32_t* rec_gid, float* rgb,
                        uint32_t* rec_score, int64_t n_total, float* score, cudaStream_t s, int bin_log2,
-                       const uint2* rec_rect);
+                       const uint2* rec_rect, uint32_t* tile_ctr, const unsigned long long* d_nvis,
+                       const uint32_t* err);
 
 // K8 / K9: adjoint of compositing and projection (fine-tuning path).
 // grec: n_rec x 9 doubles, zeroed: the adjoint sums of each record (k_backward.cu).

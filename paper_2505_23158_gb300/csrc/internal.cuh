@@ -241,6 +241,10 @@ lodge_status stream_slot(lodge_ctx* ctx, int k, Slot** out);
 // frame's stages)
 constexpr int kRenderStreams = 8;
 constexpr int kRenderStreamsFull = 3;
+// views of one importance call (six 720p views of a chunk set one after the
+// other 1775 us, on 3 / 4 / 6 streams 851 / 868 / 751; the first call of a
+// context, which makes the slots, 2050, and 1400 / 1800 / 2500)
+constexpr int kImportanceStreams = 4;
 
 // a batch of frames composited by one launch (lodge_capi.cu)
 struct BatchItem {

@@ -338,13 +338,27 @@ __global__ void __launch_bounds__(kBlendThreads, 8) blend_batch_loop_kernel(Blen
 __global__ void __launch_bounds__(kBlendThreads, 8) importance_kernel(BlendFrame f) {
     blend_tile<false, false, true>(f, blockIdx.x);
 }
+__global__ void __launch_bounds__(kBlendThreads, 8)
+importance_loop_kernel(BlendFrame f, uint32_t* __restrict__ tile_ctr) {
+    __shared__ int s_t;
+    for (;;) {
+        if (threadIdx.x == 0) s_t = (int)atomicAdd(tile_ctr, 1u);
+        __syncthreads();
+        const int t = s_t;
+        __syncthreads();   // s_t is rewritten for the next tile
+        if (t >= f.ntiles) break;
+        blend_tile<false, false, true>(f, t);
+    }
+}
 
 // raise score[gid] to each record's score
 __global__ void record_score_to_gid_kernel(const uint32_t* __restrict__ rec_score,
                                            const uint32_t* __restrict__ rec_gid, int64_t n_rec,
-                                           int64_t n_total, uint32_t* __restrict__ score) {
+                                           int64_t n_total, uint32_t* __restrict__ score,
+                                           const unsigned long long* __restrict__ d_nvis,
+                                           const uint32_t* __restrict__ err) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rec) return;
+    if (r >= n_rec || (d_nvis && (unsigned long long)r >= *d_nvis) || (*err & kErrOverflow)) return;
     const uint32_t v = rec_score[r];
     const uint32_t g = rec_gid[r];
     if (v && (int64_t)g < n_total) atomicMax(score + g, v);
@@ -438,15 +452,20 @@ void launch_importance(const DevCamera& cam, const uint2* ranges, const uint32_t
                        uint32_t vmask, int64_t n_keys, const float4* rec_a, const float4* rec_b,
                        const float* rec_c, int64_t n_rec, const uint32_t* rec_gid, float* rgb,
                        uint32_t* rec_score, int64_t n_total, float* score, cudaStream_t s, int bin_log2,
-                       const uint2* rec_rect) {
+                       const uint2* rec_rect, uint32_t* tile_ctr, const unsigned long long* d_nvis,
+                       const uint32_t* err) {
     BlendFrame f = blend_frame(cam, ranges, tile_val, vmask, n_keys, rec_a, rec_b, rec_c, n_rec,
                                BlendOut{rgb, nullptr, nullptr}, bin_log2, rec_rect);
     if (f.ntiles == 0) return;
     f.rec_score = rec_score;
-    importance_kernel<<<(unsigned)f.ntiles, kBlendThreads, 0, s>>>(f);
+    if (tile_ctr)
+        importance_loop_kernel<<<(unsigned)std::min<int64_t>(f.ntiles, (int64_t)device_sms() * kBlendCtasPerSM),
+                                 kBlendThreads, 0, s>>>(f, tile_ctr);
+    else
+        importance_kernel<<<(unsigned)f.ntiles, kBlendThreads, 0, s>>>(f);
     if (n_rec > 0)
         record_score_to_gid_kernel<<<(unsigned)((n_rec + 255) / 256), 256, 0, s>>>(
-            rec_score, rec_gid, n_rec, n_total, reinterpret_cast<uint32_t*>(score));
+            rec_score, rec_gid, n_rec, n_total, reinterpret_cast<uint32_t*>(score), d_nvis, err);
 }
 
 }  // namespace lodge

@@ -611,12 +611,12 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
                    : ctx->bin_log2 >= 0 ? ctx->bin_log2
                    : (na >= kPerTileActiveMin ? 0 : 1);
     // the key capacity is learned per bin size
-    if (!save && !importance && sl.key_cap_bl != bl) {
+    if (!save && sl.key_cap_bl != bl) {
         sl.key_cap = 0;
         sl.key_cap_bl = bl;
     }
     // no mid-frame sync: plain frames once the slot knows a key capacity
-    const bool deferred = pend && !save && !importance && !sl.prof_count &&
+    const bool deferred = pend && !save && !sl.prof_count &&
                           sl.key_cap > 0 && na > 0 && (int)sl.pending.size() < Slot::kRing;
     if (pend) pend->used = false;
     // (the stage profile's events would stand between the launches)
@@ -705,7 +705,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
             n_bkeys = (int64_t)nk64;
         }
         // capacity for later frames of this slot that skip the sync
-        if (!save && !importance)
+        if (!save)
             sl.key_cap = std::max<int64_t>(sl.key_cap, n_bkeys + n_bkeys / 2 + 65536);
     }
     const size_t nv1 = (size_t)std::max<int64_t>(n_vis, 1), nk1 = (size_t)std::max<int64_t>(n_bkeys, 1);
@@ -813,7 +813,8 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
         launch_importance(cam, ws.ranges.as<uint2>(), rec_of_pair, vmask, n_bkeys, ws.rec_a.as<float4>(),
                           ws.rec_b.as<float4>(), ws.rec_c.as<float>(), n_vis, ws.rec_gid.as<uint32_t>(),
                           d_rgb, ws.iscore.as<uint32_t>(), dsc.n_total, importance, s, bl,
-                          ws.rec_rect.as<uint2>());
+                          ws.rec_rect.as<uint2>(), sl.share_sms ? sl.d_small + kSmCtrBlend : nullptr, d_nvis,
+                          sl.d_small + kSmErr);
     } else {
         launch_blend(cam, ws.ranges.as<uint2>(), rec_of_pair, vmask, n_bkeys, ws.rec_a.as<float4>(),
                      ws.rec_b.as<float4>(), ws.rec_c.as<float>(), n_vis, bo, s, bl, ws.rec_rect.as<uint2>(),
@@ -1649,10 +1650,15 @@ static lodge_status copy_back_async(Slot& sl, float* h_dst, const float* d_src, 
 // The body of lodge_render; h_rgb != null also copies each frame's image to
 // h_rgb (same layout as d_rgb) on its slot's copy stream right after the frame,
 // so the copies of earlier frames overlap the rendering of later ones.
+// d_score != null: the frames raise the importance scores instead (their
+// images go to their slots' scratch, d_rgb is not used), over chunk `chunk`'s
+// own set if it is not negative.  The scores only grow, so that the views'
+// order does not matter.
 static lodge_status render_cams(lodge_ctx* ctx, int32_t scene_id, lodge_mode mode, const lodge_camera* cams,
                                 int32_t n_cams, float* d_rgb, void* stream, int32_t save_for_backward,
-                                int64_t* handle_out, lodge_frame_stats* stats, float* h_rgb) {
-    if (!ctx || !cams || !d_rgb || n_cams < 0) return fail(LODGE_E_INVALID, "bad argument");
+                                int64_t* handle_out, lodge_frame_stats* stats, float* h_rgb,
+                                float* d_score = nullptr, int32_t chunk = -1) {
+    if (!ctx || !cams || (!d_rgb && !d_score) || n_cams < 0) return fail(LODGE_E_INVALID, "bad argument");
     if (save_for_backward && (n_cams != 1 || !handle_out))
         return fail(LODGE_E_INVALID, "save_for_backward needs n_cams == 1 and handle_out");
     const auto t_call = std::chrono::steady_clock::now();
@@ -1669,7 +1675,9 @@ static lodge_status render_cams(lodge_ctx* ctx, int32_t scene_id, lodge_mode mod
     std::vector<Slot*> rsl{&sl0};
     std::vector<cudaStream_t> rst{s};
     if (n_cams > 1 && !save_for_backward && sc->residency == kResident) {
-        const int m = std::min<int>(mode == LODGE_FULL ? kRenderStreamsFull : kRenderStreams, n_cams);
+        const int m = std::min<int>(d_score               ? kImportanceStreams
+                                    : mode == LODGE_FULL ? kRenderStreamsFull
+                                                         : kRenderStreams, n_cams);
         for (int k = 1; k < m; ++k) {
             Slot* q = nullptr;
             TRY(stream_slot(ctx, k, &q));
@@ -1700,6 +1708,21 @@ static lodge_status render_cams(lodge_ctx* ctx, int32_t scene_id, lodge_mode mod
             q->share_sms = false;
         }
     };
+    auto frame = [&](Slot& sl, cudaStream_t si, int i, bool end_sync, Saved* sv, Slot::Pending* pd) {
+        lodge_frame_stats* st = stats ? stats + i : nullptr;
+        if (!d_score)
+            return render_one(ctx, sl, sc, mode, cams[i], d_rgb + offs[i], si, sv, st, end_sync, nullptr, pd);
+        const lodge_status r = ensure(ctx, sl.ws.img, sizeof(float) * (offs[i + 1] - offs[i]), si);
+        if (r != LODGE_OK) return r;
+        if (chunk < 0)
+            return render_one(ctx, sl, sc, mode, cams[i], sl.ws.img.as<float>(), si, nullptr, st, end_sync, d_score, pd);
+        Active act;
+        act.list = sc->chunks[chunk].list;
+        act.n = sc->chunks[chunk].n;
+        act.A = chunk;
+        return render_frame(ctx, sl, sc->dev, act, cams[i], sl.ws.img.as<float>(), si, nullptr, st, end_sync, d_score,
+                            nullptr, pd);
+    };
     for (int i = 0; i < n_cams; ++i) {
         std::unique_ptr<Saved> sv;
         if (save_for_backward) sv.reset(new Saved());
@@ -1712,9 +1735,7 @@ static lodge_status render_cams(lodge_ctx* ctx, int32_t scene_id, lodge_mode mod
         pd.frame = i;
         lodge_status r = LODGE_OK;
         if (defer && (int)sl.pending.size() >= Slot::kRing) r = harvest_front(sl, Slot::kRing / 2, &redo);
-        if (r == LODGE_OK)
-            r = render_one(ctx, sl, sc, mode, cams[i], d_rgb + offs[i], si, sv.get(),
-                           stats ? stats + i : nullptr, last, nullptr, defer ? &pd : nullptr);
+        if (r == LODGE_OK) r = frame(sl, si, i, last, sv.get(), defer ? &pd : nullptr);
         if (r != LODGE_OK) {
             drain();
             return r;
@@ -1756,8 +1777,7 @@ static lodge_status render_cams(lodge_ctx* ctx, int32_t scene_id, lodge_mode mod
     }
     for (Slot* q : rsl) q->share_sms = false;   // frames rendered again below run alone
     for (int i : redo) {
-        r = render_one(ctx, sl0, sc, mode, cams[i], d_rgb + offs[i], s, nullptr, stats ? stats + i : nullptr,
-                       true, nullptr, nullptr);
+        r = frame(sl0, s, i, true, nullptr, nullptr);
         if (r != LODGE_OK) {
             drain();
             return r;
@@ -1871,25 +1891,9 @@ lodge_status lodge_importance(lodge_ctx* ctx, int32_t scene_id, lodge_mode mode,
         if (sc->residency != kResident)
             return fail(LODGE_E_NOT_RESIDENT, "a chunk's own set is scored on resident scenes only");
     }
-    CUDA_TRY(cudaSetDevice(ctx->device));
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    Slot& sl = *ctx->slots[0];
-    for (int i = 0; i < n_cams; ++i) {
-        TRY(check_cam(cams[i]));
-        TRY(ensure(ctx, sl.ws.img, sizeof(float) * 3 * (size_t)cams[i].width * cams[i].height, s));
-        if (chunk >= 0) {
-            Active act;
-            act.list = sc->chunks[chunk].list;
-            act.n = sc->chunks[chunk].n;
-            act.A = chunk;
-            TRY(render_frame(ctx, sl, sc->dev, act, cams[i], sl.ws.img.as<float>(), s, nullptr, nullptr,
-                             true, d_score));
-        } else {
-            TRY(render_one(ctx, sl, sc, mode, cams[i], sl.ws.img.as<float>(), s, nullptr, nullptr, true,
-                           d_score));
-        }
-    }
-    return LODGE_OK;
+    for (int i = 0; i < n_cams; ++i) TRY(check_cam(cams[i]));
+    return render_cams(ctx, scene_id, mode, cams, n_cams, nullptr, stream, 0, nullptr, nullptr, nullptr, d_score,
+                       chunk);
 }
 
 // Visibility filtering (Sec. 3): keep the Gaussians of chunk `chunk` whose
