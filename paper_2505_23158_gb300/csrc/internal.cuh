@@ -234,13 +234,13 @@ lodge_status create_slot(lodge_ctx* ctx, Slot** out);
 // slot k >= 1 with its own stream (created on first use)
 lodge_status stream_slot(lodge_ctx* ctx, int k, Slot** out);
 // streams the frames of one multi-camera render call take turns on: eight
-// for chunk frames, three for full-detail frames, whose working set (the
-// whole finest level) is far larger than L2 (measured at 1080p: chunk frames
-// 5519 / 5718 / 5803 frames/s with 4 / 6 / 8 streams; full-detail frames
-// 596 / 705 with 2 / 3, their long compositing tails filled by the next
-// frame's stages)
+// for chunk frames, four for full-detail frames, whose scratch and working
+// set (the whole finest level) are far larger (chunk frames at 1080p 5519 /
+// 5718 / 5803 frames/s with 4 / 6 / 8 streams; four full-detail frames of 4M
+// Gaussians 1763 / 1556 / 1537 us with 3 / 4 / 6, twelve 307 / 304 us a frame
+// with 4 / 6, their long compositing tails filled by other frames' stages)
 constexpr int kRenderStreams = 8;
-constexpr int kRenderStreamsFull = 3;
+constexpr int kRenderStreamsFull = 4;
 // views of one importance call (six 720p views of a chunk set one after the
 // other 1775 us, on 3 / 4 / 6 streams 851 / 868 / 751; the first call of a
 // context, which makes the slots, 2050, and 1400 / 1800 / 2500)
