@@ -239,7 +239,7 @@ lodge_status lodge_set_bin_size(lodge_ctx* ctx, int32_t log2_tiles);
  * save_for_backward != 0 (n_cams must be 1) the frame's intermediate state
  * is kept under *handle_out until lodge_release.  Returns when every frame
  * has been enqueued and its counters read.  Frames of a resident scene
- * take turns on several streams (six; two for LODGE_FULL) and, once their
+ * take turns on several streams (eight; four for LODGE_FULL) and, once their
  * stream has seen a frame, run without a mid-frame synchronisation
  * (scratch sized by capacities, counts read at the end of the call); a
  * frame whose keys outgrow that capacity is rendered again
@@ -358,6 +358,13 @@ lodge_status lodge_render_params_lod(lodge_ctx* ctx, int32_t num_levels, const i
 lodge_status lodge_render_backward(lodge_ctx* ctx, int64_t handle, const float* d_dL_drgb,
                                    float* d_g_means, float* d_g_log_scales, float* d_g_quats,
                                    float* d_g_opacity_logits, float* d_g_sh, void* stream);
+
+/* The same gradients WRITTEN instead of accumulated, for every Gaussian of
+ * the trained level (0 where the frame does not show it), so that the arrays
+ * need not be zeroed first. */
+lodge_status lodge_render_gradients(lodge_ctx* ctx, int64_t handle, const float* d_dL_drgb,
+                                    float* d_g_means, float* d_g_log_scales, float* d_g_quats,
+                                    float* d_g_opacity_logits, float* d_g_sh, void* stream);
 
 /* Free a saved frame. */
 lodge_status lodge_release(lodge_ctx* ctx, int64_t handle);

@@ -116,6 +116,7 @@ _SIGS = {
     "lodge_render_params": [P, C.c_int64, P, P, P, P, P, C.c_int32, C.c_float, P, P, P,
                             C.c_int32, C.POINTER(C.c_int64), P],
     "lodge_render_backward": [P, C.c_int64, P, P, P, P, P, P, P],
+    "lodge_render_gradients": [P, C.c_int64, P, P, P, P, P, P, P],
     "lodge_release": [P, C.c_int64],
     "lodge_debug_keys": [P, C.c_int64, P, P, C.c_int64, C.POINTER(C.c_int64), P],
     "lodge_debug_records": [P, C.c_int64, P, P, P, P, P, P, P, C.c_int64,

@@ -293,6 +293,14 @@ class Lodge:
                _ptr(g_means), _ptr(g_log_scales), _ptr(g_quats), _ptr(g_logits), _ptr(g_sh),
                _stream(stream))
 
+    def render_gradients(self, handle: int, dL_drgb: torch.Tensor, g_means=None, g_log_scales=None,
+                         g_quats=None, g_logits=None, g_sh=None, stream=None):
+        """render_backward's gradients written, not accumulated: every row of
+        the given tensors is set (0 where the frame shows no such Gaussian)."""
+        A.call("lodge_render_gradients", self._h, int(handle), _ptr(dL_drgb.contiguous()),
+               _ptr(g_means), _ptr(g_log_scales), _ptr(g_quats), _ptr(g_logits), _ptr(g_sh),
+               _stream(stream))
+
     def release(self, handle: int):
         A.call("lodge_release", self._h, int(handle))
 
@@ -452,9 +460,9 @@ class _RenderParams(torch.autograd.Function):
     @staticmethod
     def backward(fctx, g_img):
         means, log_scales, quats, logits, sh = fctx.saved_tensors
-        gs = [torch.zeros_like(t) for t in (means, log_scales, quats, logits, sh)]
+        gs = [torch.empty_like(t) for t in (means, log_scales, quats, logits, sh)]
         try:
-            fctx.lodge.render_backward(fctx.handle, g_img.contiguous(), *gs)
+            fctx.lodge.render_gradients(fctx.handle, g_img.contiguous(), *gs)
         finally:
             fctx.lodge.release(fctx.handle)
         return (*gs, None, None, None, None)
@@ -480,9 +488,9 @@ class _RenderLevelLod(torch.autograd.Function):
     @staticmethod
     def backward(fctx, g_img):
         trained = fctx.saved_tensors
-        gs = [torch.zeros_like(t) for t in trained]
+        gs = [torch.empty_like(t) for t in trained]
         try:
-            fctx.lodge.render_backward(fctx.handle, g_img.contiguous(), *gs)
+            fctx.lodge.render_gradients(fctx.handle, g_img.contiguous(), *gs)
         finally:
             fctx.lodge.release(fctx.handle)
         return (*gs, None, None, None, None, None, None, None)

@@ -454,11 +454,13 @@ struct BwdLevels {
     float filter_var[kMaxLevels] = {0};
     int64_t train_lo = 0, train_hi = 0;
 };
+// fresh: the gradients of the whole trained level are written (0 where no
+// record is), not added.
 void launch_project_bwd(const DevCamera& cam, int64_t n_rec, const uint32_t* rec_gid,
                         const double* grec, const float* means, const float4* act_so,
                         const float4* act_q, const float* quats, const float* sh, int sh_degree,
                         const BwdLevels& lv, float* g_means, float* g_log_scales, float* g_quats,
-                        float* g_logits, float* g_sh, cudaStream_t s);
+                        float* g_logits, float* g_sh, bool fresh, cudaStream_t s);
 
 // SM count of the current device (queried once per device; 152 on GB300),
 // for grids sized as a multiple of the SMs

@@ -2105,9 +2105,9 @@ lodge_status lodge_render_params_lod(lodge_ctx* ctx, int32_t num_levels, const i
     return LODGE_OK;
 }
 
-lodge_status lodge_render_backward(lodge_ctx* ctx, int64_t handle, const float* d_dL_drgb, float* d_g_means,
-                                   float* d_g_log_scales, float* d_g_quats, float* d_g_opacity_logits,
-                                   float* d_g_sh, void* stream) {
+static lodge_status render_backward(lodge_ctx* ctx, int64_t handle, const float* d_dL_drgb, float* d_g_means,
+                                    float* d_g_log_scales, float* d_g_quats, float* d_g_opacity_logits,
+                                    float* d_g_sh, bool fresh, void* stream) {
     if (!ctx || !d_dL_drgb) return fail(LODGE_E_INVALID, "bad argument");
     auto it = ctx->saved.find(handle);
     if (it == ctx->saved.end()) return fail(LODGE_E_INVALID, "no saved frame %lld", (long long)handle);
@@ -2127,9 +2127,23 @@ lodge_status lodge_render_backward(lodge_ctx* ctx, int64_t handle, const float* 
                      v.last.as<uint32_t>(), d_dL_drgb, ws.grec.as<double>(), s);
     launch_project_bwd(v.cam, v.n_vis, v.rec_gid.as<uint32_t>(), ws.grec.as<double>(), v.means,
                        v.act_so.as<float4>(), v.act_q.as<float4>(), v.quats, v.sh, v.sh_degree,
-                       v.lv, d_g_means, d_g_log_scales, d_g_quats, d_g_opacity_logits, d_g_sh, s);
+                       v.lv, d_g_means, d_g_log_scales, d_g_quats, d_g_opacity_logits, d_g_sh, fresh, s);
     CUDA_TRY(cudaGetLastError());
     return sync_slot(ctx, sl, s);
+}
+
+lodge_status lodge_render_backward(lodge_ctx* ctx, int64_t handle, const float* d_dL_drgb, float* d_g_means,
+                                   float* d_g_log_scales, float* d_g_quats, float* d_g_opacity_logits,
+                                   float* d_g_sh, void* stream) {
+    return render_backward(ctx, handle, d_dL_drgb, d_g_means, d_g_log_scales, d_g_quats, d_g_opacity_logits, d_g_sh,
+                           false, stream);
+}
+
+lodge_status lodge_render_gradients(lodge_ctx* ctx, int64_t handle, const float* d_dL_drgb, float* d_g_means,
+                                    float* d_g_log_scales, float* d_g_quats, float* d_g_opacity_logits,
+                                    float* d_g_sh, void* stream) {
+    return render_backward(ctx, handle, d_dL_drgb, d_g_means, d_g_log_scales, d_g_quats, d_g_opacity_logits, d_g_sh,
+                           true, stream);
 }
 
 lodge_status lodge_release(lodge_ctx* ctx, int64_t handle) {

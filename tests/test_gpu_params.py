@@ -59,3 +59,27 @@ def test_parameter_levels_and_gradient_alignment(env, n, degree):
     for x, y in zip(ga, gb):   # the same FP64 sums of warp partials, in any order, rounded once
         assert float((x - y).abs().max()) <= 1e-6 * float(x.abs().max() + 1e-30)
     assert float(ga[4][:, 3 * (degree + 1) ** 2:].abs().sum()) == 0.0
+
+
+@pytest.mark.parametrize("n,hidden,degree", [(1, 0, 3), (33, 0, 2), (1023, 500, 1), (1024, 1024, 3), (1025, 1, 0),
+                                             (5000, 4000, 3)])
+def test_written_gradients_equal_accumulated(env, n, hidden, degree):
+    """lodge_render_gradients sets every row: the accumulated gradients where
+    a Gaussian is seen, 0 elsewhere (`hidden` ones behind the camera, in one
+    run of the list and scattered), at both alignments."""
+    torch, api, ctx = env
+    p = _params(torch, n, n, -3.0)
+    half = hidden // 2
+    p[0][:half, 2] = -50.0
+    p[0][torch.randperm(n, generator=torch.Generator().manual_seed(n))[:hidden - half].cuda(), 2] = -50.0
+    cam = _cam(90, 70)
+    img, st, h = ctx.render_params(*p, cam, sh_degree=degree, save=True)
+    w = torch.randn(img.shape, generator=torch.Generator(device="cuda").manual_seed(n), device="cuda")
+    want = [torch.zeros_like(t) for t in p]
+    ctx.render_backward(h, w, *want)
+    for shift in (0, 1):
+        got = [torch.full((t.numel() + shift,), float("nan"), device="cuda")[shift:].view(t.shape) for t in p]
+        ctx.render_gradients(h, w, *got)
+        for x, y in zip(got, want):   # the same FP64 sums of warp partials, in any order, rounded once
+            assert float((x - y).abs().max()) <= 1e-6 * float(y.abs().max() + 1e-30)
+    ctx.release(h)
