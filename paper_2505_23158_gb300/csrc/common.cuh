@@ -271,13 +271,21 @@ void launch_threshold_cost(const DevScene& sc, const DevCamera& cam, int64_t n, 
 constexpr int kSortThreads = 256;
 constexpr int kSortIPT = 15;
 constexpr int kSortTile = kSortThreads * kSortIPT;
-// inputs of at most kSortSmallMax pairs use tiles of kSortTileSmall pairs
+// inputs of at most kSortSmallMax pairs use tiles of kSortTileSmall pairs, or
+// of kSortTileShared where other frames' kernels share the SMs: the small
+// tiles fill the SMs of a lone sort (a lone chunk frame 274 us, 280 with
+// tiles of 2048), the larger ones issue fewer instructions a key (24 chunk
+// frames 3310 us with 1024, 3135 / 3108 / 3090 with 2048 / 3072 / 3840, a
+// serving step of 12 frames 1039, 1024 / 1042 / 1059)
 constexpr int kSortTileSmall = kSortThreads * 4;
+constexpr int kSortTileShared = kSortThreads * 8;
 constexpr int64_t kSortSmallMax = 1ll << 20;
-constexpr int64_t sort_tile_for(int64_t n) { return n <= kSortSmallMax ? kSortTileSmall : kSortTile; }
+constexpr int64_t sort_tile_for(int64_t n, bool shared = false) {
+    return n > kSortSmallMax ? kSortTile : shared ? kSortTileShared : kSortTileSmall;
+}
 // scratch words: 4 x 256 digit offsets, 32 tile counters, look-back words
-constexpr int64_t sort_scratch_words(int64_t n, int passes) {
-    return 4 * 256 + 32 + (int64_t)passes * ((n + sort_tile_for(n) - 1) / sort_tile_for(n)) * 256;
+constexpr int64_t sort_scratch_words(int64_t n, int passes, bool shared = false) {
+    return 4 * 256 + 32 + (int64_t)passes * ((n + sort_tile_for(n, shared) - 1) / sort_tile_for(n, shared)) * 256;
 }
 // digit_offsets: optional exclusive per-pass digit offsets (passes x 256)
 // that replace the upfront histogram; final_keys = false skips writing the
@@ -292,13 +300,13 @@ constexpr int64_t sort_scratch_words(int64_t n, int passes) {
 // scratch_cleared: the caller has zeroed the scratch (no memset here).
 // digit_counts: digit_offsets holds the per-pass digit counts instead, which
 // each pass scans itself (no separate scan launch).
-size_t sort_scratch_bytes(int64_t n, int key_bits);
+size_t sort_scratch_bytes(int64_t n, int key_bits, bool shared = false);
 int launch_onesweep(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
                     int64_t n, int key_bits, void* scratch, uint32_t* err, cudaStream_t s,
                     const uint32_t* digit_offsets = nullptr, bool final_keys = true, int shift0 = 0,
                     uint2* ranges = nullptr, uint32_t range_tiles = 0,
                     const unsigned long long* d_count = nullptr, bool scratch_cleared = false,
-                    bool digit_counts = false, bool chained = false);
+                    bool digit_counts = false, bool chained = false, bool shared = false);
 int onesweep_launches(int64_t n, int key_bits, bool offsets_supplied);
 
 // K4: emit (bin, record) pairs in depth order.  A bin is a square of

@@ -239,16 +239,20 @@ uint32_t last_mask_for(int key_bits) {
     return last_bits >= 8 ? 0xffu : ((1u << last_bits) - 1u);
 }
 
-constexpr int kSmallIPT = kSortTileSmall / kSortThreads;
-static_assert(kSmallIPT * kSortThreads == kSortTileSmall, "small tile must be whole items per thread");
+constexpr int kSmallIPT = kSortTileSmall / kSortThreads, kSharedIPT = kSortTileShared / kSortThreads;
+static_assert(kSmallIPT * kSortThreads == kSortTileSmall && kSharedIPT * kSortThreads == kSortTileShared,
+              "tiles must be whole items per thread");
 
 template <bool kWK, bool kV>
-void launch_pass(bool small, int64_t ntiles, const uint32_t* ki, const uint32_t* vi, uint32_t* ko,
+void launch_pass(int64_t tile, int64_t ntiles, const uint32_t* ki, const uint32_t* vi, uint32_t* ko,
                  uint32_t* vo, int64_t n, int shift, uint32_t dm, const uint32_t* off, uint32_t* st,
                  uint32_t* ctr, uint32_t* err, uint2* ranges, int range_shift, uint32_t range_tiles,
                  const unsigned long long* d_count, bool raw, cudaStream_t s, bool chained) {
-    if (small)
+    if (tile == kSortTileSmall)
         launch_chained(chained, onesweep_pass<kSmallIPT, kWK, kV>, (unsigned)ntiles, kSortThreads, s, ki, vi, ko, vo,
+                       n, shift, dm, off, st, ctr, err, ranges, range_shift, range_tiles, d_count, raw);
+    else if (tile == kSortTileShared)
+        launch_chained(chained, onesweep_pass<kSharedIPT, kWK, kV>, (unsigned)ntiles, kSortThreads, s, ki, vi, ko, vo,
                        n, shift, dm, off, st, ctr, err, ranges, range_shift, range_tiles, d_count, raw);
     else
         launch_chained(chained, onesweep_pass<kSortIPT, kWK, kV>, (unsigned)ntiles, kSortThreads, s, ki, vi, ko, vo,
@@ -257,20 +261,20 @@ void launch_pass(bool small, int64_t ntiles, const uint32_t* ki, const uint32_t*
 
 }  // namespace
 
-size_t sort_scratch_bytes(int64_t n, int key_bits) {
-    return sizeof(uint32_t) * (size_t)sort_scratch_words(n, passes_for(key_bits));
+size_t sort_scratch_bytes(int64_t n, int key_bits, bool shared) {
+    return sizeof(uint32_t) * (size_t)sort_scratch_words(n, passes_for(key_bits), shared);
 }
 
 int launch_onesweep(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
                     int64_t n, int key_bits, void* scratch, uint32_t* err, cudaStream_t s,
                     const uint32_t* digit_offsets, bool final_keys, int shift0, uint2* ranges,
                     uint32_t range_tiles, const unsigned long long* d_count, bool scratch_cleared,
-                    bool digit_counts, bool chained) {
+                    bool digit_counts, bool chained, bool shared) {
     const int P = passes_for(key_bits);
     if (P == 0 || (d_count ? n < 1 : n <= 1)) return 0;
     if (d_count && !digit_offsets) return 0;   // device counts need supplied digit offsets
-    const bool small = sort_tile_for(n) == kSortTileSmall;
-    const int64_t ntiles = (n + sort_tile_for(n) - 1) / sort_tile_for(n);
+    const int64_t tile = sort_tile_for(n, shared);
+    const int64_t ntiles = (n + tile - 1) / tile;
     const bool values = vals != nullptr;
     uint32_t* hist = static_cast<uint32_t*>(scratch);
     uint32_t* counters = hist + kMaxPasses * kRadix;
@@ -283,10 +287,10 @@ int launch_onesweep(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t
         // exclusive digit offsets supplied: clear only counters and look-back words
         if (!scratch_cleared)
             cudaMemsetAsync(counters, 0,
-                            sort_scratch_bytes(n, key_bits) - sizeof(uint32_t) * kMaxPasses * kRadix, s);
+                            sort_scratch_bytes(n, key_bits, shared) - sizeof(uint32_t) * kMaxPasses * kRadix, s);
         offs = digit_offsets;
     } else {
-        cudaMemsetAsync(scratch, 0, sort_scratch_bytes(n, key_bits), s);
+        cudaMemsetAsync(scratch, 0, sort_scratch_bytes(n, key_bits, shared), s);
         int hist_blocks = (int)std::min<int64_t>((n + 255) / 256, (int64_t)device_sms() * 4);
         hist_kernel<<<hist_blocks, 256, 0, s>>>(keys, n, P, last_mask, hist, shift0);
         hist_scan_kernel<<<P, kRadix, 0, s>>>(hist);
@@ -299,10 +303,10 @@ int launch_onesweep(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t
         const int sh = shift0 + 8 * p;
         uint2* rg = p == P - 1 ? ranges : nullptr;
         if (values) {
-            if (wk) launch_pass<true, true>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
-            else launch_pass<false, true>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
+            if (wk) launch_pass<true, true>(tile, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
+            else launch_pass<false, true>(tile, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
         } else {
-            launch_pass<true, false>(small, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
+            launch_pass<true, false>(tile, ntiles, ki, vi, ko, vo, n, sh, dm, offs + p * kRadix, stp, counters + p, err, rg, shift0, range_tiles, d_count, raw, s, chained);
         }
         std::swap(ki, ko);
         std::swap(vi, vo);

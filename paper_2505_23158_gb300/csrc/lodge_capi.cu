@@ -632,16 +632,16 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
         // counters and look-back words, the bin ranges (begin ~0, end 0)
         const int64_t etiles = std::max<int64_t>(emit_tiles(na, kEmitThreads), 1);
         TRY(ensure(ctx, ws.status2, sizeof(uint32_t) * (size_t)etiles, s));
-        TRY(ensure(ctx, ws.sort, sort_scratch_bytes(na, 32), s));
-        TRY(ensure(ctx, ws.sort2, sort_scratch_bytes(sl.key_cap, tbits), s));
+        TRY(ensure(ctx, ws.sort, sort_scratch_bytes(na, 32, sl.share_sms), s));
+        TRY(ensure(ctx, ws.sort2, sort_scratch_bytes(sl.key_cap, tbits, sl.share_sms), s));
         TRY(ensure(ctx, ws.ranges, sizeof(uint2) * (size_t)std::max<int64_t>(nbins, 1), s));
         FillPlan fp;
         fp.add(ws.status.as<uint32_t>(), ptiles);
         fp.add(sl.d_small, kSmWords);
         fp.add(ws.doffs.as<uint32_t>(), 8 * 256);
         fp.add(ws.status2.as<uint32_t>(), etiles);
-        fp.add(ws.sort.as<uint32_t>(), (int64_t)(sort_scratch_bytes(na, 32) / sizeof(uint32_t)));
-        fp.add(ws.sort2.as<uint32_t>(), (int64_t)(sort_scratch_bytes(sl.key_cap, tbits) / sizeof(uint32_t)));
+        fp.add(ws.sort.as<uint32_t>(), (int64_t)(sort_scratch_bytes(na, 32, sl.share_sms) / sizeof(uint32_t)));
+        fp.add(ws.sort2.as<uint32_t>(), (int64_t)(sort_scratch_bytes(sl.key_cap, tbits, sl.share_sms) / sizeof(uint32_t)));
         fp.add(reinterpret_cast<uint32_t*>(ws.ranges.p), 2 * nbins, 0xffffffffu, 0u);
         int64_t most = 0;
         for (int k = 0; k < fp.count; ++k) most = std::max(most, fp.n[k]);
@@ -714,12 +714,12 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     TRY(ensure(ctx, ws.dkey2, sizeof(uint32_t) * nv1, s));
     TRY(ensure(ctx, ws.dval2, sizeof(uint32_t) * nv1, s));
     if (!deferred)   // (frames without a sync set up their own sort scratch above)
-        TRY(ensure(ctx, ws.sort, std::max(sort_scratch_bytes(n_vis, 32), sort_scratch_bytes(n_bkeys, tbits)), s));
+        TRY(ensure(ctx, ws.sort, std::max(sort_scratch_bytes(n_vis, 32, sl.share_sms), sort_scratch_bytes(n_bkeys, tbits, sl.share_sms)), s));
     prof_begin(sl, LODGE_STAGE_DEPTH_SORT, s);
     // (the passes scan the projection's digit counts themselves)
     int w1 = launch_onesweep(ws.dkey.as<uint32_t>(), ws.dval.as<uint32_t>(), ws.dkey2.as<uint32_t>(),
                              ws.dval2.as<uint32_t>(), n_vis, 32, ws.sort.p, sl.d_small + kSmErr, s,
-                             po.depth_hist, true, 0, nullptr, 0, d_nvis, deferred, true, chained);
+                             po.depth_hist, true, 0, nullptr, 0, d_nvis, deferred, true, chained, sl.share_sms);
     prof_end(sl, LODGE_STAGE_DEPTH_SORT, s, onesweep_launches(n_vis, 32, true));
     DBuf& zs = w1 ? ws.dkey2 : ws.dkey;
     DBuf& rs = w1 ? ws.dval2 : ws.dval;
@@ -777,7 +777,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
                              tbits, deferred ? ws.sort2.p : ws.sort.p, sl.d_small + kSmErr, s,
                              ws.doffs.as<uint32_t>(), true, rbits,
                              fused_ranges ? ws.ranges.as<uint2>() : nullptr, (uint32_t)nbins, d_nbk, deferred,
-                             true, chained);   // (the emission leaves its digit counts unscanned)
+                             true, chained, sl.share_sms);   // (the emission leaves its digit counts unscanned)
     prof_end(sl, LODGE_STAGE_TILE_SORT, s, onesweep_launches(n_bkeys, tbits, true));
     DBuf& ks = w2 ? ws.tkey2 : ws.tkey;
     DBuf& vs = w2 ? ws.tval2 : ws.tval;
