@@ -24,8 +24,9 @@
 //   skip if alpha < 1/255; T' = T (1 - alpha); stop if T' < 1e-4;
 //   C += T alpha rgb; T = T'.
 // The step has no branches: alpha becomes 0 where the pixel skips (T' = T,
-// weight 0) and T becomes 0 where it stops, which makes every later step a
-// no-op.  A thread's two pixels run in packed FP32 pairs.
+// weight 0); a pixel that stops keeps its T' < 1e-4, which makes the weight
+// of every later step 0 (T only falls).  A thread's two pixels run in packed
+// FP32 pairs.
 //
 // What bounds it: instruction issue and the FP32 pipes.  A visit of a record
 // by a warp (64 pixels) takes about 38 instructions, 30 FP32 pipe cycles of
@@ -36,8 +37,13 @@
 // 858k records 455 -> 254 us, its longest lists being walked four records at
 // a time instead of one after the other.  Storing the scalars that enter
 // packed steps twice in shared memory measured no fewer FP32 instructions (a
-// packed operand may be one register used twice).  64 registers (8 CTAs per
+// packed operand may be one register used twice).  A list's last one to three
+// records are visited as a pair and a single (filling the turn up with a
+// record that nothing composites, and zeroing a stopped pixel's T: lone
+// chunk frame 276 against 270 us, four 4K frames 1298 against 1276).  64 registers (8 CTAs per
 // SM): 10 CTAs with 48 measured 2-4% slower, no limit (66-72 registers) 1-3%.
+#include <type_traits>
+
 #include "walk.cuh"
 
 namespace lodge {
@@ -47,7 +53,8 @@ namespace {
 constexpr int kBlendThreads = 128; // blend: two pixels per thread
 constexpr int kBlendBatch = 128;   // blend: records per batch (one per thread)
 constexpr int kUnroll = 4;         // records visited per turn of the walk
-constexpr uint32_t kNoHit = 16u * kBlendBatch;   // offset of a record no pixel composites
+
+constexpr float kStop = 1e-4f;      // a pixel stops before its transmittance falls below
 
 // two pixels of one thread
 struct PixelPair {
@@ -63,11 +70,11 @@ __device__ __forceinline__ f32x2 keep2(bool lo, bool hi, f32x2 a, f32x2 b) {
 }
 
 // One record against the thread's two pixels (Eq. 1).  Returns the weights
-// T alpha (0 where the pixel skips or has stopped) and the transmittances
-// after the record (0 where it has stopped).
+// T alpha (0 where the pixel skips or has stopped); T becomes the
+// transmittance after the record (below kStop where it has stopped).
 __device__ __forceinline__ void blend_pair(const char* __restrict__ rec, float pxf, float py0, PixelPair& p,
                                            f32x2& wgt) {
-    constexpr int kNext = sizeof(float4) * (kBlendBatch + 1);
+    constexpr int kNext = sizeof(float4) * kBlendBatch;
     const float4 a = *reinterpret_cast<const float4*>(rec);
     const float4 b = *reinterpret_cast<const float4*>(rec + kNext);
     const float cz = *reinterpret_cast<const float*>(rec + 2 * kNext);
@@ -82,9 +89,8 @@ __device__ __forceinline__ void blend_pair(const char* __restrict__ rec, float p
     const f32x2 Tn = mul2(p.T, fma2(al, pack2(-1.f, -1.f), pack2(1.f, 1.f)));
     float n0, n1;
     unpack2(Tn, n0, n1);
-    const f32x2 go = pack2(ge01(n0, 1e-4f), ge01(n1, 1e-4f));
-    wgt = mul2(mul2(p.T, al), go);
-    p.T = mul2(Tn, go);
+    wgt = mul2(mul2(p.T, al), pack2(ge01(n0, kStop), ge01(n1, kStop)));
+    p.T = Tn;
     p.C0 = fma2(wgt, pack2(b.z, b.z), p.C0);
     p.C1 = fma2(wgt, pack2(b.w, b.w), p.C1);
     p.C2 = fma2(wgt, pack2(cz, cz), p.C2);
@@ -97,10 +103,10 @@ __device__ __forceinline__ void blend_pair(const char* __restrict__ rec, float p
 template <bool kSave, bool kCount = false, bool kScore = false>
 __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
     __shared__ uint32_t s_id[kScore ? 2 : 1][kScore ? kBlendBatch : 1];   // staged records
-    __shared__ uint32_t s_top[kScore ? kBlendBatch + 1 : 1];              // their largest weights here
-    __shared__ float4 s_rec[2][3][kBlendBatch + 1];        // the last one composites nowhere
+    __shared__ uint32_t s_top[kScore ? kBlendBatch : 1];                  // their largest weights here
+    __shared__ float4 s_rec[2][3][kBlendBatch];
     __shared__ uint32_t s_met[4][kBlendBatch / 32];        // per block: which records reach it
-    __shared__ __align__(8) uint16_t s_hit[4][kBlendBatch + kUnroll];   // per warp: their offsets
+    __shared__ __align__(8) uint16_t s_hit[4][kBlendBatch];   // per warp: their offsets
     const int32_t width = f.width, height = f.height, tiles_x = f.tiles_x;
     const uint32_t* __restrict__ tile_val = f.tile_val;
     const uint32_t vmask = f.vmask, n_keys = f.n_keys, n_rec = f.n_rec;
@@ -132,7 +138,7 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
     auto stopped = [&]() {
         float T0, T1;
         unpack2(p.T, T0, T1);
-        return T0 == 0.f && T1 == 0.f;
+        return T0 < kStop && T1 < kStop;
     };
     auto stage = [&](int buf, uint32_t key) {
         const uint32_t j = min(key & vmask, n_rec - 1u);
@@ -142,12 +148,7 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
         cp_async4(&s_rec[buf][2][tid].x, rec_c + j);
         cp_async8(&s_rec[buf][2][tid].z, rec_rect + j);
     };
-    if (tid < 2) {   // alpha = 2^-inf = 0
-        s_rec[tid][0][kBlendBatch] = make_float4(0.f, 0.f, 0.f, 0.f);
-        s_rec[tid][1][kBlendBatch] = make_float4(0.f, __int_as_float(0x7f800000), 0.f, 0.f);
-        s_rec[tid][2][kBlendBatch] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    if (kScore) s_top[tid] = 0u;   // (the last one is read, never raised)
+    if (kScore) s_top[tid] = 0u;
     if (tid < n) stage(0, tile_val[tid]);
     cp_async_commit();
     uint32_t key = kBlendBatch + tid < n ? tile_val[kBlendBatch + tid] : 0u;
@@ -185,20 +186,29 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
                     s_hit[warp][nh + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(16 * (w * 32 + lane));
                 nh += __popc(m);
             }
-            if (lane < kUnroll) s_hit[warp][nh + lane] = (uint16_t)kNoHit;
             __syncwarp();
             const char* base = reinterpret_cast<const char*>(&s_rec[buf][0][0]);
-            for (int i = 0; i < nh; i += kUnroll) {
-                const uint2 h = *reinterpret_cast<const uint2*>(&s_hit[warp][i]);
-                const uint32_t off[kUnroll] = {h.x & 0xffffu, h.x >> 16, h.y & 0xffffu, h.y >> 16};
-                uint32_t top = 0u, top_at = 0u;   // lane u: largest weight of the turn's record u
+            // the next kN records of the list, together
+            auto visit = [&](auto count, int i) {
+                constexpr int kN = decltype(count)::value;
+                uint32_t off[kN];
+                if (kN == kUnroll) {
+                    const uint2 h = *reinterpret_cast<const uint2*>(&s_hit[warp][i]);
+                    off[0] = h.x & 0xffffu; off[1 % kN] = h.x >> 16; off[2 % kN] = h.y & 0xffffu; off[3 % kN] = h.y >> 16;
+                } else if (kN == 2) {
+                    const uint32_t h = *reinterpret_cast<const uint32_t*>(&s_hit[warp][i]);
+                    off[0] = h & 0xffffu; off[1 % kN] = h >> 16;
+                } else {
+                    off[0] = s_hit[warp][i];
+                }
+                uint32_t top = 0u, top_at = 0u;   // lane u: largest weight of record u
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
+                for (int u = 0; u < kN; ++u) {
                     f32x2 wgt;
-                    if (kCount && off[u] != kNoHit) {
+                    if (kCount) {
                         float T0, T1;
                         unpack2(p.T, T0, T1);
-                        n_eval += (T0 > 0.f ? 1u : 0u) + (T1 > 0.f ? 1u : 0u);
+                        n_eval += (T0 < kStop ? 0u : 1u) + (T1 < kStop ? 0u : 1u);
                     }
                     const PixelPair before = p;
                     blend_pair(base + off[u], pxf, py0, p, wgt);
@@ -223,7 +233,16 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
                     }
                 }
                 if (kScore && top > s_top[top_at]) atomicMax(&s_top[top_at], top);
+            };
+            int i = 0;
+            for (; i + kUnroll <= nh; i += kUnroll) {
+                visit(std::integral_constant<int, kUnroll>{}, i);
                 if (__all_sync(0xffffffffu, stopped())) break;
+            }
+            // the list's end, without visits that composite nothing
+            if (i + kUnroll > nh) {
+                if (nh & 2) { visit(std::integral_constant<int, 2>{}, i); i += 2; }
+                if (nh & 1) visit(std::integral_constant<int, 1>{}, i);
             }
         }
         const bool end = __syncthreads_count(stopped()) == kBlendThreads;
