@@ -192,9 +192,14 @@ __device__ __forceinline__ bool key_splat(const DevScene& sc, const DevCamera& c
     return true;
 }
 
-// six CTAs per SM (at most 42 registers): the kernel is bound by the
-// latency of its dependent gathers, so resident warps matter more than the
-// few spilled words
+// Eight CTAs per SM (32 registers): the kernel is bound by the latency of its
+// dependent gathers, so resident warps matter more than the spilled words
+// (lone chunk frame 267 us at six, 262.5 at eight, LOD frame 271 and 262, 24
+// chunk frames 3118 and 3057; CTAs of 128 threads: lone 260, but four
+// full-detail frames 1545 -> 1690, twice the look-back links).  kRaw and
+// kBlocks, whose sources take more registers, stay at six (fine-tuning step
+// 1480, 1510 at eight).  The visible ones are counted by ballots and one
+// barrier.
 //
 // kRaw reads the caller's parameter arrays where they lie.  Activating them
 // into a store first (a transpose of the 192-byte SH rows above all, of every
@@ -202,11 +207,11 @@ __device__ __forceinline__ bool key_splat(const DevScene& sc, const DevCamera& c
 // before a projection of 110 us for 2M Gaussians, 58% of them visible; this
 // one takes 135 us alone.
 template <int kSrc>
-__global__ void __launch_bounds__(kProjThreads, 6)
+__global__ void __launch_bounds__(kProjThreads, kSrc == kStore ? 8 : 6)
 project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict__ tile_counter,
                uint32_t* __restrict__ err) {
     __shared__ uint32_t s_tile, s_prefix;
-    __shared__ uint32_t s_scan[33];
+    __shared__ uint32_t s_cnt[kProjThreads / 32];
     __shared__ unsigned long long s_keys, s_bkeys;
     __shared__ uint32_t s_dh[4][256];   // depth-key digit counts (the depth sort's histogram)
     if (P.o.depth_hist)
@@ -304,8 +309,16 @@ project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict
     // count is published as soon as it is known and the look-back comes
     // after the attribute work below, so successors rarely wait on it and
     // this CTA's own look-back finds its predecessors' counts in place.
-    uint32_t total;
-    uint32_t excl = block_exclusive_scan(vis ? 1u : 0u, s_scan, &total);
+    const uint32_t seen = __ballot_sync(0xffffffffu, vis);
+    if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = (uint32_t)__popc(seen);
+    __syncthreads();
+    uint32_t total = 0, excl = (uint32_t)__popc(seen & ((1u << (threadIdx.x & 31)) - 1u));
+#pragma unroll
+    for (int w = 0; w < kProjThreads / 32; ++w) {
+        const uint32_t c = s_cnt[w];
+        if (w < (int)(threadIdx.x >> 5)) excl += c;
+        total += c;
+    }
     if (threadIdx.x == 0) st_volatile(status + tile, (tile == 0 ? kStInc : kStAgg) | total);
     uint32_t nk = vis ? (rx1 - rx0 + 1) * (ry1 - ry0 + 1) : 0u;
     {
