@@ -186,14 +186,16 @@ struct ResidencyStats {
 struct lodge_ctx {
     int device = 0;
     size_t budget = 0;
-    // Scratch and saved frames come from the context's own pool, which keeps
-    // freed memory mapped while it holds at most kPoolKeep bytes in all (none
-    // when a budget is set; given back when an allocation fails): a
-    // training step saves its frame's buffers and frees them after the
-    // adjoint, and the device's default pool unmaps freed memory at every
+    // Scratch and saved frames come from one pool that a device's contexts
+    // without a budget share.  It keeps freed memory mapped while it holds at
+    // most kPoolKeep bytes in all, gives it back when an allocation fails and
+    // is destroyed with its last context: a training step saves its frame's
+    // buffers and frees them after the adjoint, and the device's default pool
+    // (which contexts with a budget use) unmaps freed memory at every
     // synchronisation, so that each step mapped it anew.  A fine-tuning step
     // of 2M Gaussians at 720p: 2427 -> 2192 us.
     cudaMemPool_t pool = nullptr;
+    bool pool_shared = false;
     size_t used = 0;                 // device bytes held; guarded by mu
     std::recursive_mutex mu;         // budget, blocks, saved frames, slot list
     std::condition_variable_any freed;  // signalled when device memory is released

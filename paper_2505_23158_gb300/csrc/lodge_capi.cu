@@ -91,6 +91,52 @@ bool make_room(lodge_ctx* ctx, size_t bytes) {
     return true;
 }
 
+// the pool that the contexts of a device share, and how many they are
+struct SharedPool {
+    cudaMemPool_t pool = nullptr;
+    int refs = 0;
+};
+constexpr int kMaxPools = 64;
+static SharedPool g_pools[kMaxPools];
+static std::mutex g_pools_mu;
+
+static cudaError_t acquire_pool(lodge_ctx* ctx) {
+    if (ctx->budget || ctx->device >= kMaxPools) return cudaDeviceGetDefaultMemPool(&ctx->pool, ctx->device);
+    std::lock_guard<std::mutex> lk(g_pools_mu);
+    SharedPool& sp = g_pools[ctx->device];
+    if (!sp.pool) {
+        cudaMemPoolProps pp{};
+        pp.allocType = cudaMemAllocationTypePinned;
+        pp.location.type = cudaMemLocationTypeDevice;
+        pp.location.id = ctx->device;
+        uint64_t keep = kPoolKeep;
+        cudaError_t e = cudaMemPoolCreate(&sp.pool, &pp);
+        if (e == cudaSuccess) {
+            e = cudaMemPoolSetAttribute(sp.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) cudaMemPoolDestroy(sp.pool);
+        }
+        if (e != cudaSuccess) {
+            sp.pool = nullptr;
+            return e;
+        }
+    }
+    ++sp.refs;
+    ctx->pool = sp.pool;
+    ctx->pool_shared = true;
+    return cudaSuccess;
+}
+
+static void release_pool(lodge_ctx* ctx) {
+    if (!ctx->pool_shared) return;
+    std::lock_guard<std::mutex> lk(g_pools_mu);
+    SharedPool& sp = g_pools[ctx->device];
+    if (--sp.refs == 0) {
+        cudaMemPoolDestroy(sp.pool);
+        sp.pool = nullptr;
+    }
+    ctx->pool_shared = false;
+}
+
 bool trim_pool(lodge_ctx* ctx) {
     cudaGetLastError();
     return cudaDeviceSynchronize() == cudaSuccess && cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess;
@@ -1293,15 +1339,13 @@ lodge_status lodge_create(int device, size_t hbm_budget_bytes, lodge_ctx** out) 
     fill_qtable_host(q);
     CUDA_TRY(upload_qtable(q));
     CUDA_TRY(cudaStreamCreateWithFlags(&ctx->upload_stream, cudaStreamNonBlocking));
-    cudaMemPoolProps pp{};
-    pp.allocType = cudaMemAllocationTypePinned;
-    pp.location.type = cudaMemLocationTypeDevice;
-    pp.location.id = device;
-    CUDA_TRY(cudaMemPoolCreate(&ctx->pool, &pp));
-    uint64_t keep = hbm_budget_bytes ? 0 : kPoolKeep;
-    CUDA_TRY(cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    CUDA_TRY(acquire_pool(ctx.get()));
     Slot* s0 = nullptr;
-    TRY(create_slot(ctx.get(), &s0));
+    const lodge_status r = create_slot(ctx.get(), &s0);
+    if (r != LODGE_OK) {
+        release_pool(ctx.get());
+        return r;
+    }
     *out = ctx.release();
     return LODGE_OK;
 }
@@ -1317,7 +1361,7 @@ lodge_status lodge_destroy(lodge_ctx* ctx) {
     for (auto& sl : ctx->slots) destroy_slot(ctx, *sl);
     if (ctx->upload_stream) cudaStreamDestroy(ctx->upload_stream);
     cudaDeviceSynchronize();
-    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+    release_pool(ctx);
     delete ctx;
     return LODGE_OK;
 }
