@@ -1,6 +1,7 @@
 """What the compositing's adjoint works out in FP32: partial sums over at most
-32 pixels before they are added in FP64.  The test is built so that the exact
-value is known; the bar is derived beside it."""
+32 pixels before they are added in FP64, and the transmittance restored by
+IEEE quotients.  Each test is built so that the exact value is known; the bars
+are derived beside it."""
 import numpy as np
 import pytest
 
@@ -69,3 +70,31 @@ def test_partials_span_32_pixels(env):
     want = float(Y0) * 64 * float(np.float32(0.99))
     # FP32 roundings after the sum: its cast and the product with Y0
     assert abs(float(gs[4][0, 0]) - want) <= 2 * 2.0 ** -24 * want
+
+
+# logits of two splats on the pixel's centre and their alphas on the device
+@pytest.mark.parametrize("l1,l2,a1,a2", [
+    ("-0x1.8331cp-1", "-0x1.d553dp+1", "0x1.472168p-2", "0x1.98615ap-6"),
+    ("-0x1.5296cp+0", "-0x1.affe28p+1", "0x1.aeddcp-3", "0x1.0f0e1ap-5"),
+    ("0x1.781c9p+0", "-0x1.cad6fp+1", "0x1.a038d4p-1", "0x1.ba4f1ap-6"),
+    ("-0x1.ff5638p+1", "-0x1.71af4p+1", "0x1.28307p-6", "0x1.b00fd4p-5"),
+    ("0x1.bb198p-2", "-0x1.8869a4p+1", "0x1.368a02p-1", "0x1.6ce666p-5")])
+def test_transmittance_restored_by_ieee_quotients(env, l1, l2, a1, a2):
+    """The colour gradient that one pixel gives the splat behind is Y0 T alpha
+    with T = T_final / (1 - alpha), each operation rounded as IEEE has it (the
+    bar is equality).  An approximate quotient with one remainder correction
+    is off by a unit in the last place for these pairs."""
+    torch, ctx = env
+    l1, l2, a1, a2 = (np.float32(float.fromhex(x)) for x in (l1, l2, a1, a2))
+    one = np.float32(1)
+    ps = _stack(torch, [l1, l2], -12.0, (0.5, 0.5, 0.5))
+    g = torch.zeros(17, 17, 3)
+    g[8, 8, 0] = 1.0
+    img, gs = _render(ctx, torch, ps, _cam(17, 17), g)
+    T1 = one - a1
+    T2 = T1 * (one - a2)
+    want = (np.float64(a1) * 0.5 + np.float64(T1 * a2) * 0.5).astype(np.float32)   # the alphas are as given
+    assert np.float32(float(img[8, 8, 0])) == want
+    T = T2 / (one - a2)
+    assert np.float32(float(gs[4][1, 0])) == Y0 * (T * a2)
+    assert np.float32(float(gs[4][0, 0])) == Y0 * ((T / (one - a1)) * a1)
