@@ -505,6 +505,11 @@ lodge_status lodge_residency_stats(lodge_ctx* ctx, lodge_residency* out);
  * device. */
 lodge_status lodge_inject_upload_failures(lodge_ctx* ctx, int32_t n);
 
+/* Fault injection for tests: the next n frames report a device-side wait that
+ * gave up (LODGE_E_TIMEOUT from the call that renders them).  Their kernels
+ * run as ever; the frame's status word is set after the last one. */
+lodge_status lodge_inject_frame_timeouts(lodge_ctx* ctx, int32_t n);
+
 /* ---------------------------------------------------------------- profiling */
 
 /* Stages of a frame, in launch order. */

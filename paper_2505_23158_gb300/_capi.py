@@ -127,6 +127,7 @@ _SIGS = {
     "lodge_serve": [P, P, C.c_int32, C.POINTER(lodge_serve_opts), P],
     "lodge_residency_stats": [P, C.POINTER(lodge_residency)],
     "lodge_inject_upload_failures": [P, C.c_int32],
+    "lodge_inject_frame_timeouts": [P, C.c_int32],
     "lodge_set_bin_size": [P, C.c_int32],
     "lodge_profile_enable": [P, C.c_int],
     "lodge_profile_read": [P, C.POINTER(lodge_profile)],

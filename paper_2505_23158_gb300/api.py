@@ -399,6 +399,10 @@ class Lodge:
     def inject_upload_failures(self, n: int):
         A.call("lodge_inject_upload_failures", self._h, int(n))
 
+    def inject_frame_timeouts(self, n: int):
+        """The next n frames report a wait that gave up (tests)."""
+        A.call("lodge_inject_frame_timeouts", self._h, int(n))
+
     def profile_enable(self, enable: bool = True, count_pairs: bool = False):
         """Event timing per stage (counters reset); count_pairs: the counting
         mode (compositing counts its pixel-Gaussian pairs; times not plain)."""

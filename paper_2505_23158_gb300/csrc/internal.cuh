@@ -3,6 +3,7 @@
 // request loop).
 #pragma once
 
+#include <atomic>
 #include <condition_variable>
 #include <map>
 #include <memory>
@@ -209,6 +210,7 @@ struct lodge_ctx {
     cudaStream_t upload_stream = nullptr;
     lodge::ResidencyStats res;
     int fail_next_uploads = 0;       // host-side fault injection
+    std::atomic<int> fail_next_frames{0};
     int bin_log2 = -1;               // key lists per bin of 2^bin_log2 x 2^bin_log2 tiles (-1: by frame)
 };
 

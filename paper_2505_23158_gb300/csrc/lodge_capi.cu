@@ -399,6 +399,14 @@ static Scene* get_scene(lodge_ctx* ctx, int32_t id) {
     return ctx->scenes[id].get();
 }
 
+// a frame's status word as the call's outcome
+static lodge_status status_of(uint32_t err) {
+    if (err & kErrTimeout) return fail(LODGE_E_TIMEOUT, "a device-side wait timed out (status 0x%x)", err);
+    if (err & kErrOverflow) return fail(LODGE_E_OVERFLOW, "device output capacity exceeded (status 0x%x)", err);
+    if (err & kErrBadIndex) return fail(LODGE_E_INVALID, "out-of-range index in an active list (status 0x%x)", err);
+    return LODGE_OK;
+}
+
 lodge_status sync_slot(lodge_ctx* ctx, Slot& sl, cudaStream_t s) {
     (void)ctx;
     CUDA_TRY(cudaMemcpyAsync(sl.h_small, sl.d_small, sizeof(uint32_t) * kSmWords,
@@ -410,10 +418,7 @@ lodge_status sync_slot(lodge_ctx* ctx, Slot& sl, cudaStream_t s) {
         err |= sl.h_tail[kSmErr];
         sl.tail_pending = false;
     }
-    if (err & kErrTimeout) return fail(LODGE_E_TIMEOUT, "a device-side wait timed out (status 0x%x)", err);
-    if (err & kErrOverflow) return fail(LODGE_E_OVERFLOW, "device output capacity exceeded (status 0x%x)", err);
-    if (err & kErrBadIndex) return fail(LODGE_E_INVALID, "out-of-range index in an active list (status 0x%x)", err);
-    return LODGE_OK;
+    return status_of(err);
 }
 
 // ---------------------------------------------------------------------------
@@ -870,6 +875,10 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
     }
     prof_end(sl, LODGE_STAGE_BLEND, s, job ? 0 : ntiles_img > 0 ? (importance ? 1 + (n_vis > 0) : 1) : 0);
     CUDA_TRY(cudaGetLastError());
+    if (ctx->fail_next_frames.load(std::memory_order_relaxed) > 0 && ctx->fail_next_frames.fetch_sub(1) > 0) {
+        // (injected: the status word of a wait that gave up)
+        CUDA_TRY(cudaMemsetAsync(sl.d_small + kSmErr, kErrTimeout, 1, s));
+    }
     if (deferred) {
         // status words and counts into the slot's ring; read at its harvest
         const int ring = sl.ring_next;
@@ -952,17 +961,22 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
 }
 
 // Wait for a slot's stream and take the status words and counts of its
-// deferred frames (stats, profile).  A frame whose bin keys outgrew the
+// deferred frames (stats, profile), and the status word of a frame before
+// them whose end was not waited for.  A frame whose bin keys outgrew the
 // slot's capacity wrote no keys: the capacity grows and the frame's index is
 // appended to *redo, to be rendered again with its mid-frame sync.
 static void take_pending(Slot& sl, const Slot::Pending& p, std::vector<int>* redo, lodge_status* r);
 
 static lodge_status harvest(lodge_ctx* ctx, Slot& sl, cudaStream_t s, std::vector<int>* redo) {
     (void)ctx;
-    if (sl.pending.empty()) return LODGE_OK;
+    if (sl.pending.empty() && !sl.tail_pending) return LODGE_OK;
     CUDA_TRY(cudaStreamSynchronize(s));
     prof_collect(sl);
     lodge_status r = LODGE_OK;
+    if (sl.tail_pending) {
+        sl.tail_pending = false;
+        r = status_of(sl.h_tail[kSmErr]);
+    }
     for (const Slot::Pending& p : sl.pending) take_pending(sl, p, redo, &r);
     sl.pending.clear();
     return r;
@@ -1001,10 +1015,7 @@ static void take_pending(Slot& sl, const Slot::Pending& p, std::vector<int>* red
         if (redo) redo->push_back(p.frame);
         return;
     }
-    if (r == LODGE_OK && (err & kErrTimeout))
-        r = fail(LODGE_E_TIMEOUT, "a device-side wait timed out (status 0x%x)", err);
-    if (r == LODGE_OK && (err & kErrBadIndex))
-        r = fail(LODGE_E_INVALID, "out-of-range index in an active list (status 0x%x)", err);
+    if (r == LODGE_OK) r = status_of(err);
     sl.prof.frames += 1;
     sl.prof.keys += (int64_t)nk;
     sl.prof.bin_keys += (int64_t)nb;
@@ -2332,6 +2343,12 @@ lodge_status lodge_set_bin_size(lodge_ctx* ctx, int32_t log2_tiles) {
     if (!ctx || log2_tiles < -1 || log2_tiles > 3) return fail(LODGE_E_INVALID, "bad argument");
     std::lock_guard<std::recursive_mutex> lk(ctx->mu);
     ctx->bin_log2 = log2_tiles;
+    return LODGE_OK;
+}
+
+lodge_status lodge_inject_frame_timeouts(lodge_ctx* ctx, int32_t n) {
+    if (!ctx || n < 0) return fail(LODGE_E_INVALID, "bad argument");
+    ctx->fail_next_frames = n;
     return LODGE_OK;
 }
 
