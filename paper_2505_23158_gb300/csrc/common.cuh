@@ -312,7 +312,8 @@ int onesweep_launches(int64_t n, int key_bits, bool offsets_supplied);
 // K4: emit (bin, record) pairs in depth order.  A bin is a square of
 // 2^bin_log2 x 2^bin_log2 tiles (bin_log2 = 0: the 16x16 tile itself), bins_x
 // per image row; a record goes to every bin its tile rect touches.  koff:
-// n_vis + 1 words; srec / srect: n_vis gathered record ids and bin rects;
+// n_vis + 1 words; srec / srect: n_vis gathered record ids and bin rects (all
+// three used where emit_by_record only, null elsewhere);
 // n_keys (bin keys) from the projection's count.  digit_hist (zeroed,
 // 4 x 256 words) receives the bin sort's digit counts on key_bits bin bits,
 // not scanned (launch_onesweep with digit_counts scans them).  rbits > 0: one packed word per pair,
@@ -329,6 +330,10 @@ __host__ __device__ __forceinline__ int64_t emit_tiles(int64_t n, int rest) {
     return kEmitNear / kEmitNearTile + (n - kEmitNear + rest - 1) / rest;
 }
 constexpr int64_t kEmitWarpMinKeys = 32;  // mean keys per record for one warp per record
+// whether launch_emit takes one warp per record (with koff, srec and srect)
+inline bool emit_by_record(int64_t n_vis, int64_t n_keys) {
+    return n_vis > 0 && n_keys >= kEmitWarpMinKeys * n_vis;
+}
 int launch_emit(const uint32_t* sorted_rec, int64_t n_vis, const uint2* rec_rect,
                 int32_t bins_x, int bin_log2, uint32_t* koff, uint32_t* srec, uint2* srect,
                 int64_t n_keys, uint32_t* tile_key, uint32_t* tile_val, int rbits, int key_bits,

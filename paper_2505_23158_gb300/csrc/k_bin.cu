@@ -484,7 +484,7 @@ int launch_emit(const uint32_t* sorted_rec, int64_t n_vis, const uint2* rec_rect
                 uint32_t* digit_hist, uint32_t* status, uint32_t* tile_counter, uint32_t* err,
                 cudaStream_t s) {
     if (n_vis == 0 || n_keys == 0) return 0;
-    if (n_keys < kEmitWarpMinKeys * n_vis)
+    if (!emit_by_record(n_vis, n_keys))
         return launch_emit_counted(sorted_rec, n_vis, nullptr, rec_rect, bins_x, bin_log2, n_keys, nullptr,
                                    tile_key, tile_val, rbits, key_bits, digit_hist, status, tile_counter, err, s);
     // records average a warp's worth of keys or more: one warp per record

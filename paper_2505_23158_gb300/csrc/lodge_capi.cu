@@ -787,9 +787,11 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
         TRY(ensure(ctx, ws.tval, sizeof(uint32_t) * nk1, s));
         TRY(ensure(ctx, ws.tval2, sizeof(uint32_t) * nk1, s));
     }
-    TRY(ensure(ctx, ws.koff, sizeof(uint32_t) * (nv1 + 1), s));
-    TRY(ensure(ctx, ws.srec, sizeof(uint32_t) * nv1, s));
-    TRY(ensure(ctx, ws.srect, sizeof(uint2) * nv1, s));
+    if (!deferred && emit_by_record(n_vis, n_bkeys)) {   // (16 bytes a record that no other emission reads)
+        TRY(ensure(ctx, ws.koff, sizeof(uint32_t) * (nv1 + 1), s));
+        TRY(ensure(ctx, ws.srec, sizeof(uint32_t) * nv1, s));
+        TRY(ensure(ctx, ws.srect, sizeof(uint2) * nv1, s));
+    }
     if (!deferred) {
         const int64_t etiles = std::max<int64_t>(emit_tiles(n_vis, kEmitThreads), 1);
         TRY(ensure(ctx, ws.status, sizeof(uint32_t) * (size_t)etiles, s));
