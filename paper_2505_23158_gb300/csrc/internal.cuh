@@ -155,6 +155,9 @@ struct Slot {
     // other slots' frames run at the same time (several render streams, the
     // request loop): compositing then leaves room on every SM for them
     bool share_sms = false;
+    // calls that use the slot now (SlotHold), guarded by the context's mu; the
+    // scratch of a slot without one may be given back (drop_idle_scratch)
+    int in_use = 0;
     int64_t uploads = 0;       // chunk blocks this slot's frames have gathered
     lodge_profile prof{};
     cudaEvent_t ev_beg[LODGE_NUM_STAGES] = {};
@@ -226,11 +229,36 @@ lodge_status dmalloc(lodge_ctx* ctx, void** p, size_t bytes);
 void dfree(lodge_ctx* ctx, void* p, size_t bytes);
 lodge_status ensure(lodge_ctx* ctx, DBuf& b, size_t bytes, cudaStream_t s);
 void release(lodge_ctx* ctx, DBuf& b, cudaStream_t s);
-// the pool's freed memory back to the device, after an allocation failed
-bool trim_pool(lodge_ctx* ctx);
-// evict unreferenced blocks (least recently used first) until `bytes` more
-// fit in the budget; caller holds ctx->mu; returns false if they cannot
+// the scratch of the slots that no call uses freed (slot 0, which the
+// single-frame calls use, excepted): a call on several streams leaves it
+// behind.  Whether there was any.  Caller holds ctx->mu.
+bool drop_idle_scratch(lodge_ctx* ctx);
+// idle scratch and the pool's freed memory back to the device, after an
+// allocation failed; caller holds ctx->mu
+bool give_back(lodge_ctx* ctx);
+// evict unreferenced blocks (least recently used first), then idle scratch,
+// until `bytes` more fit in the budget; caller holds ctx->mu; returns false
+// if they cannot
 bool make_room(lodge_ctx* ctx, size_t bytes);
+
+// Slots 1 and up that a call uses.  It must have waited for their streams
+// before it lets go of them.
+struct SlotHold {
+    explicit SlotHold(lodge_ctx* c) : ctx(c) {}
+    ~SlotHold() { let_go(); }
+    void add(Slot* sl) {
+        std::lock_guard<std::recursive_mutex> lk(ctx->mu);
+        ++sl->in_use;
+        held.push_back(sl);
+    }
+    void let_go() {
+        std::lock_guard<std::recursive_mutex> lk(ctx->mu);
+        for (Slot* sl : held) --sl->in_use;
+        held.clear();
+    }
+    lodge_ctx* ctx;
+    std::vector<Slot*> held;
+};
 
 lodge_status sync_slot(lodge_ctx* ctx, Slot& sl, cudaStream_t s);
 const char* last_error();

@@ -80,7 +80,10 @@ bool make_room(lodge_ctx* ctx, size_t bytes) {
                 key = kv.first;
             }
         }
-        if (!victim) return false;
+        if (!victim) {
+            if (drop_idle_scratch(ctx)) continue;
+            return false;
+        }
         // the block is unreferenced: every frame that read it has completed
         cudaFreeAsync(victim->mem, ctx->upload_stream);
         if (victim->ready) cudaEventDestroy(victim->ready);
@@ -137,8 +140,25 @@ static void release_pool(lodge_ctx* ctx) {
     ctx->pool_shared = false;
 }
 
-bool trim_pool(lodge_ctx* ctx) {
+// (no work is in flight on an idle slot)
+bool drop_idle_scratch(lodge_ctx* ctx) {
+    size_t bytes = 0;
+    for (auto& slp : ctx->slots) {
+        if (slp->index == 0 || slp->in_use) continue;
+        for (DBuf* b : slp->ws.all()) {
+            if (!b->p) continue;
+            cudaFreeAsync(b->p, ctx->upload_stream);
+            bytes += b->cap;
+            *b = DBuf{};
+        }
+    }
+    ctx->used -= bytes;
+    return bytes > 0;
+}
+
+bool give_back(lodge_ctx* ctx) {
     cudaGetLastError();
+    drop_idle_scratch(ctx);
     return cudaDeviceSynchronize() == cudaSuccess && cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess;
 }
 
@@ -148,7 +168,7 @@ lodge_status dmalloc(lodge_ctx* ctx, void** p, size_t bytes) {
         return fail(LODGE_E_BUDGET, "HBM budget exceeded: %zu in use + %zu requested > %zu",
                     ctx->used, bytes, ctx->budget);
     cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaErrorMemoryAllocation && trim_pool(ctx)) e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && give_back(ctx)) e = cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(LODGE_E_OOM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
@@ -186,7 +206,7 @@ lodge_status ensure(lodge_ctx* ctx, DBuf& b, size_t bytes, cudaStream_t s) {
         b.cap = 0;
     }
     cudaError_t e = cudaMallocFromPoolAsync(&b.p, ncap, ctx->pool, s);
-    if (e == cudaErrorMemoryAllocation && trim_pool(ctx)) e = cudaMallocFromPoolAsync(&b.p, ncap, ctx->pool, s);
+    if (e == cudaErrorMemoryAllocation && give_back(ctx)) e = cudaMallocFromPoolAsync(&b.p, ncap, ctx->pool, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         b.p = nullptr;
@@ -1067,7 +1087,11 @@ lodge_status render_one(lodge_ctx* ctx, Slot& sl, Scene* sc, lodge_mode mode,
 lodge_status render_batch(lodge_ctx* ctx, BatchItem* items, int n, int first, cudaStream_t s) {
     if (n < 1 || n > kMaxBlendBatch) return fail(LODGE_E_INVALID, "batch of %d frames (1..%d)", n, kMaxBlendBatch);
     std::vector<Slot*> q((size_t)n);
-    for (int k = 0; k < n; ++k) TRY(stream_slot(ctx, first + k, &q[k]));
+    SlotHold hold(ctx);
+    for (int k = 0; k < n; ++k) {
+        TRY(stream_slot(ctx, first + k, &q[k]));
+        hold.add(q[k]);
+    }
     std::vector<BlendFrame> jobs;
     std::vector<int> ok;
     std::vector<Slot::Pending> pd((size_t)n);
@@ -1731,20 +1755,24 @@ static lodge_status render_cams(lodge_ctx* ctx, int32_t scene_id, lodge_mode mod
     // stream ends after all of it.
     std::vector<Slot*> rsl{&sl0};
     std::vector<cudaStream_t> rst{s};
+    SlotHold hold(ctx);
     if (n_cams > 1 && !save_for_backward && sc->residency == kResident) {
         const int m = std::min<int>(d_score               ? kImportanceStreams
                                     : mode == LODGE_FULL ? kRenderStreamsFull
                                                          : kRenderStreams, n_cams);
         for (int k = 1; k < m; ++k) {
             Slot* q = nullptr;
-            TRY(stream_slot(ctx, k, &q));
+            const lodge_status r = stream_slot(ctx, k, &q);
+            if (r == LODGE_E_BUDGET || r == LODGE_E_OOM) break;
+            if (r != LODGE_OK) return r;
+            hold.add(q);
             CUDA_TRY(cudaEventRecord(q->fence, s));
             CUDA_TRY(cudaStreamWaitEvent(q->own, q->fence, 0));
             rsl.push_back(q);
             rst.push_back(q->own);
         }
     }
-    const int m = (int)rsl.size();
+    int m = (int)rsl.size();
     for (Slot* q : rsl) q->share_sms = m > 1;
     // Frames of a resident scene that are not kept for the adjoint run
     // without their mid-frame sync once their slot knows a key capacity:
@@ -1758,12 +1786,34 @@ static lodge_status render_cams(lodge_ctx* ctx, int32_t scene_id, lodge_mode mod
     auto drain = [&]() {   // after a failure: nothing of this call stays in flight
         for (int k = 0; k < m; ++k) {
             Slot* q = rsl[k];
-            if (q->tail_pending || !q->pending.empty()) cudaStreamSynchronize(rst[k]);
+            cudaStreamSynchronize(rst[k]);
             if (h_rgb && q->copy) cudaStreamSynchronize(q->copy);
             q->tail_pending = false;
             q->pending.clear();
             q->share_sms = false;
         }
+    };
+    // No memory for a frame while several slots hold scratch: the frames so far
+    // are waited for, the other slots' scratch is given back, and the call goes
+    // on with slot 0 alone, as a call of one frame after another would.
+    auto to_one_slot = [&]() {
+        lodge_status r = LODGE_OK;
+        for (int k = 0; k < m; ++k) {
+            Slot* q = rsl[k];
+            const cudaError_t e = cudaStreamSynchronize(rst[k]);
+            if (r == LODGE_OK && e != cudaSuccess) r = fail(LODGE_E_CUDA, "%s", cudaGetErrorString(e));
+            if (r == LODGE_OK) r = harvest(ctx, *q, rst[k], &redo);
+            if (h_rgb && q->copy) cudaStreamSynchronize(q->copy);
+            q->share_sms = false;
+        }
+        if (r != LODGE_OK) return r;
+        hold.let_go();
+        rsl.resize(1);
+        rst.resize(1);
+        m = 1;
+        std::lock_guard<std::recursive_mutex> lk(ctx->mu);
+        drop_idle_scratch(ctx);
+        return LODGE_OK;
     };
     auto frame = [&](Slot& sl, cudaStream_t si, int i, bool end_sync, Saved* sv, Slot::Pending* pd) {
         lodge_frame_stats* st = stats ? stats + i : nullptr;
@@ -1793,6 +1843,13 @@ static lodge_status render_cams(lodge_ctx* ctx, int32_t scene_id, lodge_mode mod
         lodge_status r = LODGE_OK;
         if (defer && (int)sl.pending.size() >= Slot::kRing) r = harvest_front(sl, Slot::kRing / 2, &redo);
         if (r == LODGE_OK) r = frame(sl, si, i, last, sv.get(), defer ? &pd : nullptr);
+        if (m > 1 && (r == LODGE_E_BUDGET || r == LODGE_E_OOM)) {
+            r = to_one_slot();
+            if (r == LODGE_OK) {
+                --i;   // this frame again, on slot 0
+                continue;
+            }
+        }
         if (r != LODGE_OK) {
             drain();
             return r;

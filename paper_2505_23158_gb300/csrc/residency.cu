@@ -182,7 +182,7 @@ lodge_status acquire_block(lodge_ctx* ctx, Slot& sl, Scene* sc, int chunk, cudaS
                             "(%zu of %zu in use, the rest held by frames in flight)",
                             chunk, sc->id, b->bytes, ctx->used, ctx->budget);
             cudaError_t e = cudaMallocAsync(&b->mem, b->bytes, ctx->upload_stream);
-            if (e == cudaErrorMemoryAllocation && trim_pool(ctx))
+            if (e == cudaErrorMemoryAllocation && give_back(ctx))
                 e = cudaMallocAsync(&b->mem, b->bytes, ctx->upload_stream);
             if (e != cudaSuccess) {
                 cudaGetLastError();

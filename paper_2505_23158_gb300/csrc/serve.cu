@@ -40,8 +40,10 @@ extern "C" lodge_status lodge_serve(lodge_ctx* ctx, const lodge_request* reqs, i
         lodge_status r = create_slot(ctx, &sl);
         if (r != LODGE_OK) return r;
     }
+    SlotHold hold(ctx);
     for (int w = 1; w <= need; ++w) {   // slots made by lodge_render_batch have no stream yet
         Slot& sl = *ctx->slots[w];
+        hold.add(&sl);
         sl.share_sms = opts->slots > 1;   // requests run side by side
         if (!sl.own) {
             e = cudaStreamCreateWithFlags(&sl.own, cudaStreamNonBlocking);
@@ -166,6 +168,7 @@ extern "C" lodge_status lodge_serve(lodge_ctx* ctx, const lodge_request* reqs, i
         for (int w = 1; w <= opts->slots; ++w) th.emplace_back(worker, w);
         for (auto& t : th) t.join();
     }
+    for (int w = 1; w <= need; ++w) cudaStreamSynchronize(ctx->slots[w]->own);   // (a failed frame's kernels)
     if (failures.load() > 0)
         return fail(LODGE_E_INVALID, "%d of %d requests failed (see their status)", failures.load(), n);
     return LODGE_OK;

@@ -51,3 +51,60 @@ def test_scratch_of_a_frame(env):
     depth = 4 * 4 + 4                                   # keys and records twice, look-back words of 4 passes
     key = 4 * 2 + 2                                     # packed twice, look-back words of at most 2 passes
     assert used <= 1.25 * ((record + depth) * n + key * cap) + (1 << 20)
+
+
+@pytest.mark.parametrize("call", ["importance", "importance_chunk", "full", "chunk_blend", "lod"])
+def test_several_streams_in_the_memory_of_one(env, call):
+    """A list of cameras in a context whose budget holds the scene and the
+    scratch of one frame at a time: the images and scores are those of the
+    cameras one by one."""
+    torch, api = env
+    scene, cams = synth.workload_outdoor(seed=6, n_poses=40, scale=0.05, width=320, height_px=180)
+    cams = cams[::4]
+    mode = {"importance": api.FULL, "full": api.FULL, "lod": api.LOD}.get(call, api.CHUNK_BLEND)
+
+    def run(ctx, sid, cs):
+        if call == "importance":
+            return ctx.importance(sid, mode, cs)
+        if call == "importance_chunk":
+            return ctx.importance(sid, api.CHUNK, cs, chunk=1)
+        out = torch.empty(len(cs), 180, 320, 3, device="cuda")
+        return torch.stack(ctx.render(sid, mode, cs, out=out.view(-1))[0])
+
+    with api.Lodge(0) as ctx:
+        sid = ctx.load_scene(scene)
+        want = [run(ctx, sid, [c]) for c in cams for _ in range(2)][::2]
+        alone = ctx.residency_stats()["hbm_used"]
+        run(ctx, sid, cams)
+        assert ctx.residency_stats()["hbm_used"] > 1.05 * alone    # several streams hold more
+    want = torch.stack(want).amax(0) if call.startswith("importance") else torch.cat(want)
+    budget = alone + (1 << 16)
+    with api.Lodge(0, hbm_budget_bytes=budget) as ctx:
+        sid = ctx.load_scene(scene)
+        for _ in range(2):
+            assert torch.equal(run(ctx, sid, cams), want)
+            assert ctx.residency_stats()["hbm_used"] <= budget
+
+
+def test_scratch_left_behind_is_given_back(env):
+    """The scratch that a call over several views leaves on its streams' slots
+    yields to what the context needs next."""
+    torch, api = env
+    a, b = _scene(60_000), _scene(200_000, seed=1)
+    cams = [_cam(160, 120, 0.05 * i) for i in range(6)]
+    with api.Lodge(0) as ctx:
+        sid = ctx.load_scene(a)
+        base = ctx.residency_stats()["hbm_used"]
+        want = torch.stack([ctx.importance(sid, api.FULL, [c]) for c in cams for _ in range(2)]).amax(0)
+        one = ctx.residency_stats()["hbm_used"]
+        ctx.importance(sid, api.FULL, cams)
+        several = ctx.residency_stats()["hbm_used"]
+        ctx.load_scene(b)
+        scene_b = ctx.residency_stats()["hbm_used"] - several
+    assert several - one < 0.9 * scene_b                    # the budget below holds the slots' scratch at first
+    with api.Lodge(0, hbm_budget_bytes=one + int(1.05 * scene_b)) as ctx:
+        sid = ctx.load_scene(a)
+        assert torch.equal(ctx.importance(sid, api.FULL, cams), want)
+        assert ctx.residency_stats()["hbm_used"] > base + 1.5 * (one - base)
+        ctx.load_scene(b)
+        assert torch.equal(ctx.importance(sid, api.FULL, cams), want)
