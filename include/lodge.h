@@ -388,6 +388,12 @@ lodge_status lodge_debug_records(lodge_ctx* ctx, int64_t handle, uint32_t* d_gid
                                  float* d_opacity, float* d_rgb, int64_t cap,
                                  int64_t* n_visible, void* stream);
 
+/* Image of a saved frame (width * height * 3 floats) by a plain walk: every
+ * record of the tile's list at every pixel, in order, one operation after the
+ * other.  The frames themselves skip records that cannot reach a block of
+ * pixels; they give this image bit for bit. */
+lodge_status lodge_debug_composite(lodge_ctx* ctx, int64_t handle, float* d_rgb, void* stream);
+
 /* Sort n (key, value) pairs of 32-bit unsigned integers by the key bits
  * [0, key_bits), stably, with the library's onesweep LSD radix sort.
  * d_keys/d_vals are sorted in place (device).  Exposed for testing the sort

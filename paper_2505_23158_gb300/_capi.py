@@ -118,6 +118,7 @@ _SIGS = {
     "lodge_render_backward": [P, C.c_int64, P, P, P, P, P, P, P],
     "lodge_render_gradients": [P, C.c_int64, P, P, P, P, P, P, P],
     "lodge_release": [P, C.c_int64],
+    "lodge_debug_composite": [P, C.c_int64, P, P],
     "lodge_debug_keys": [P, C.c_int64, P, P, C.c_int64, C.POINTER(C.c_int64), P],
     "lodge_debug_records": [P, C.c_int64, P, P, P, P, P, P, P, C.c_int64,
                             C.POINTER(C.c_int64), P],

@@ -341,6 +341,12 @@ class Lodge:
                _ptr(r["rgb"]), n.value, C.byref(n), _stream(stream))
         return {k: v[:n.value] for k, v in r.items()}
 
+    def debug_composite(self, handle: int, height: int, width: int, stream=None):
+        """A saved frame's image by a plain walk over its tiles' lists."""
+        img = torch.empty(height, width, 3, device=f"cuda:{self.device}")
+        A.call("lodge_debug_composite", self._h, int(handle), _ptr(img), _stream(stream))
+        return img
+
     # -- serving and residency
     def serve(self, requests, slots: int = 4, realtime: bool = True, images: bool = False,
               wait_limit_s: float = 10.0, batch: int = 0):

@@ -1233,6 +1233,39 @@ __global__ void debug_records_kernel(int64_t n, const float4* ra, const float4* 
     if (rgb) { rgb[3 * i] = b.z; rgb[3 * i + 1] = b.w; rgb[3 * i + 2] = rc[i]; }
 }
 
+// Eq. 1 over a tile's whole list, one thread per pixel, scalar: the reference
+// of the filtered walks.  A pixel takes t and w from the row pair that its
+// thread of the compositing has (rows y and y + 4 of an 8-row block).
+__global__ void debug_composite_kernel(DevCamera cam, const uint2* ranges, const uint32_t* tile_val, uint32_t vmask,
+                                       uint32_t n_keys, uint32_t n_rec, const float4* ra, const float4* rb,
+                                       const float* rc, float* out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)cam.width * cam.height) return;
+    const int x = (int)(i % cam.width), y = (int)(i / cam.width);
+    uint2 rg = ranges[(y / kTile) * cam.tiles_x + x / kTile];
+    if (rg.y > n_keys || rg.x > rg.y) rg = make_uint2(0, 0);
+    float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
+    for (uint32_t k = rg.x; k < rg.y; ++k) {
+        const uint32_t j = min(tile_val[k] & vmask, n_rec - 1u);
+        const float4 a = ra[j], b = rb[j];
+        float t0, w0, t1, w1;
+        row_pair_tw(a, b, (float)x + 0.5f - a.x, (float)(y & ~4) + 0.5f, t0, w0, t1, w1);
+        const float t = (y & 4) ? t1 : t0, w = (y & 4) ? w1 : w0;
+        const float alpha = fminf(0.99f, ex2_approx(-fmaf(t, t, fmaf(w, w, b.y))));
+        if (!(alpha >= 1.0f / 255.0f)) continue;
+        const float Tn = T * (1.f - alpha);
+        if (Tn < 1e-4f) break;
+        const float wgt = T * alpha;
+        C0 = fmaf(wgt, b.z, C0);
+        C1 = fmaf(wgt, b.w, C1);
+        C2 = fmaf(wgt, rc[j], C2);
+        T = Tn;
+    }
+    out[3 * i] = C0;
+    out[3 * i + 1] = C1;
+    out[3 * i + 2] = C2;
+}
+
 // N x 3 means -> planes, for the level selection of a parameter frame
 __global__ void planes_kernel(int64_t n, const float* means, float* mx, float* my, float* mz) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2318,6 +2351,23 @@ lodge_status lodge_debug_records(lodge_ctx* ctx, int64_t handle, uint32_t* d_gid
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaStreamSynchronize(s));
     release(ctx, zrec, s);
+    return LODGE_OK;
+}
+
+lodge_status lodge_debug_composite(lodge_ctx* ctx, int64_t handle, float* d_rgb, void* stream) {
+    if (!ctx || !d_rgb) return fail(LODGE_E_INVALID, "bad argument");
+    auto it = ctx->saved.find(handle);
+    if (it == ctx->saved.end()) return fail(LODGE_E_INVALID, "no saved frame %lld", (long long)handle);
+    CUDA_TRY(cudaSetDevice(ctx->device));
+    const Saved& v = *it->second;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const int64_t npix = (int64_t)v.cam.width * v.cam.height;
+    debug_composite_kernel<<<(unsigned)((npix + 127) / 128), 128, 0, s>>>(
+        v.cam, v.ranges.as<uint2>(), v.rbits ? v.tkey.as<uint32_t>() : v.tval.as<uint32_t>(),
+        v.rbits ? (1u << v.rbits) - 1u : 0xffffffffu, (uint32_t)v.n_keys, (uint32_t)std::max<int64_t>(v.n_vis, 1),
+        v.rec_a.as<float4>(), v.rec_b.as<float4>(), v.rec_c.as<float>(), d_rgb);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaStreamSynchronize(s));
     return LODGE_OK;
 }
 
