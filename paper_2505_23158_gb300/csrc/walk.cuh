@@ -61,34 +61,47 @@ __device__ __forceinline__ float ge01(float a, float b) {
 // bottom left, 3: bottom right; (tx0, ty0) the tile's first pixel) a record
 // can reach with alpha >= 1/255 at a pixel centre.
 //
-// The record's pixel rect must meet the block, and its ellipse must reach
-// one of the block's pixel centres: with d = p - mean' and q(d) = (u00 dx +
-// u01 dy)^2 + (u11 dy)^2 (the exponent's quadratic, a convex function with
-// its minimum 0 at d = 0), the least q over the box of the block's pixel
-// centres [X, X + 7] x [Y, Y + 7] lies on the line dx = xc or on dy = yc,
+// The record's tile rect must hold the tile (which the lists of coarser bins
+// leave open), and its ellipse must reach the box of the block's pixel
+// centres: with d = p - mean' and q(d) = (u00 dx + u01 dy)^2 + (u11 dy)^2 (the
+// exponent's quadratic, a convex function with its minimum 0 at d = 0), the
+// least q over the box [X, X + 7] x [Y, Y + 7] lies on dx = xc or on dy = yc,
 // where xc, yc are the box coordinates nearest the mean (0 where the box
 // spans it): along each line q is a one-dimensional quadratic whose minimiser
 // (dy = -u00 u01 xc / (u01^2 + u11^2), dx = -u01 yc / u00) is clamped to the
 // box.  A pixel centre can pass the 1/255 skip only if q <= log2 o' + log2
-// 255; the test adds a margin of 0.01 (in log2 units) for the rounding of q,
-// so it never drops a record that some pixel of the block would composite.
+// 255 <= 8; the test adds a margin for the rounding of q, so it never drops a
+// record that some pixel of the block would composite.  The covariance is at
+// least 0.3 I, so that u00^2 and u01^2 + u11^2 are at most 2.41 and the terms
+// of t and w at most M = 2.2 (max|dx| + max|dy|) over the tile; t and w, each
+// a few roundings of them here and in the walk, differ by at most d = 11 eps M
+// (eps = 2^-24), so that q differs by at most 2 sqrt(8) sqrt(2) d + 2 d^2 <=
+// 5.3e-6 M + 9e-13 M^2.  With s = |dx| + |dy| at the tile's first pixel, M <=
+// 2.2 (s + 30).  (s passes 1000 only where a splat of that many pixels reaches
+// the tile from afar.  With a fixed margin of 0.01, one block in 3e5 lost a
+// record of 3e5 pixels and one in ten one of 1e7.)
 //
 // One thread tests its record against all four blocks: the reciprocals are
 // the record's, the clamped x terms a column's and the y terms a row's, so
 // that four tests cost about 80 operations instead of 45 each.
 //
-// kNan: a record whose form is not a number (a covariance that overflows
-// FP32) is kept, as in a walk without the test; the plain frames drop it.
-template <bool kNan>
+// kSaved (frames kept for the adjoint, the adjoint, scores): a record whose
+// form is not a number (a covariance that overflows FP32) is kept, as in a
+// walk without the test.  The plain frames drop it, and a record whose pixel
+// rect misses the block: the rect holds the pixel centres within the extent,
+// so a splat smaller than a pixel often misses a block that its ellipse, tested
+// over the whole box of the centres, meets (four full-detail frames of 4M
+// Gaussians 1540 us, 1575 without).  The rect's margin, 0.1% of the exponent,
+// covers the rounding of the mean's coordinate up to some thousand pixels.
+template <bool kSaved>
 __device__ __forceinline__ uint32_t blocks_met(const float4 a, const float4 b, const uint2 rect, uint32_t tx0,
                                                uint32_t ty0) {
     constexpr float kLog2_255 = 7.99435343f;
     const uint32_t rx0 = rect.x & 0xffffu, ry0 = rect.x >> 16, rx1 = rect.y & 0xffffu, ry1 = rect.y >> 16;
     if (rx0 > tx0 + 15u || rx1 < tx0 || ry0 > ty0 + 15u || ry1 < ty0) return 0u;
-    const bool cx[2] = {rx0 <= tx0 + 7u, rx1 >= tx0 + 8u};
-    const bool cy[2] = {ry0 <= ty0 + 7u, ry1 >= ty0 + 8u};
+    const bool cx[2] = {kSaved || rx0 <= tx0 + 7u, kSaved || rx1 >= tx0 + 8u};
+    const bool cy[2] = {kSaved || ry0 <= ty0 + 7u, kSaved || ry1 >= ty0 + 8u};
     const float u00 = a.z, u01 = a.w, u11 = b.x;
-    const float lim = (kLog2_255 + 0.01f) - b.y;   // b.y = -log2 o'
     const float iy = __fdividef(-u00 * u01, fmaf(u01, u01, u11 * u11));
     const float ix = __fdividef(-u01, u00);
     float X0[2], X1[2], Y0[2], Y1[2], ym[2], ux[2], xm[2], uy[2], wy[2];
@@ -106,6 +119,8 @@ __device__ __forceinline__ uint32_t blocks_met(const float4 a, const float4 b, c
         const float w = u11 * yc;
         wy[k] = w * w;
     }
+    const float s = fabsf(X0[0]) + fabsf(Y0[0]);
+    const float lim = fmaf(s, fmaf(5e-12f, s, 1.6e-5f), (kLog2_255 + 0.011f) - b.y);   // b.y = -log2 o'
     uint32_t met = 0;
 #pragma unroll
     for (int r = 0; r < 2; ++r)
@@ -116,7 +131,7 @@ __device__ __forceinline__ uint32_t blocks_met(const float4 a, const float4 b, c
             const float dx = fminf(fmaxf(xm[r], X0[c]), X1[c]);
             const float t2 = fmaf(u00, dx, uy[r]);
             const float q = fminf(fmaf(t1, t1, w1 * w1), fmaf(t2, t2, wy[r]));
-            if (cx[c] && cy[r] && (kNan ? !(q > lim) : q <= lim)) met |= 1u << (2 * r + c);
+            if (cx[c] && cy[r] && (kSaved ? !(q > lim) : q <= lim)) met |= 1u << (2 * r + c);
         }
     return met;
 }

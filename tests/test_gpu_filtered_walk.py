@@ -78,3 +78,35 @@ def test_thin_rotated_splats_at_the_threshold(env, seed, wh):
                      np.log(o / (1 - o)).astype(np.float32), r.normal(0, 0.3, (n, 16, 3)).astype(np.float32))
     img, st = _check(torch, ctx, _params(torch, lv), cam)
     assert st["n_visible"] > n // 4 and float(img.max()) > 0.05
+
+
+@pytest.mark.parametrize("seed,pixels", [(4, (3e3, 3e4)), (5, (3e4, 1e6)), (6, (1e6, 3e7))])
+def test_splats_that_reach_the_image_from_afar(env, seed, pixels):
+    """Splats of up to 3e7 pixels, a few pixels wide, whose means lie up to two
+    standard deviations off the image along their long axis: the terms of the
+    exponent are then far larger than the exponent, and its rounding larger
+    than any fixed margin."""
+    torch, ctx = env
+    r = np.random.default_rng(seed)
+    n, w, h = 4000, 61, 45
+    cam = synth.look_at((0.0, 0.0, 0.0), (0.0, 0.0, 1.0), (0.0, -1.0, 0.0), w, h, 60.0)
+    R, t = np.asarray(cam.R, np.float64), np.asarray(cam.t, np.float64)
+    sigma = np.exp(r.uniform(*np.log(pixels), n))           # standard deviation along the axis, pixels
+    th = r.uniform(0, np.pi, n)
+    along = r.uniform(-2.0, 2.0, n) * sigma
+    px = r.uniform(0, w, n) + along * np.cos(th)
+    py = r.uniform(0, h, n) + along * np.sin(th)
+    z = r.uniform(1.0, 3.0, n)
+    p = np.stack([(px - cam.cx) / cam.fx * z, (py - cam.cy) / cam.fy * z, z], 1)
+    means = (p - t) @ R
+    axis = np.stack([np.cos(th), np.sin(th), 0 * th], 1) @ R    # in the image plane: world direction
+    phi = np.arctan2(axis[:, 1], axis[:, 0])
+    assert np.abs(axis[:, 2]).max() < 1e-6                      # the camera looks along z
+    logs = np.log(np.stack([sigma, np.exp(r.uniform(np.log(0.01), np.log(3), n)), np.full(n, 1e-3)], 1)
+                  * (z / cam.fx)[:, None])
+    quats = np.stack([np.cos(phi / 2), 0 * phi, 0 * phi, np.sin(phi / 2)], 1)
+    o = np.exp(r.uniform(np.log(1.02 / 255), np.log(5 / 255), n))
+    lv = synth.Level(means.astype(np.float32), logs.astype(np.float32), quats.astype(np.float32),
+                     np.log(o / (1 - o)).astype(np.float32), r.normal(0, 0.3, (n, 16, 3)).astype(np.float32))
+    img, st = _check(torch, ctx, _params(torch, lv), cam)
+    assert st["n_visible"] > n // 4 and float(img.max()) > 0.05
