@@ -30,7 +30,9 @@ constexpr uint32_t kSpinFast = 64;          // polls before a wait starts to sle
 // there is room, and wait at chain_wait until that kernel has completed with
 // its writes visible (as it waited for its own predecessor, so has everything
 // before).  Every kernel of the chain calls chain_wait before it touches
-// global memory.  Both calls do nothing in a launch that is not chained.
+// global memory, and its pointers carry no __restrict__: the kernel before it
+// still writes their targets after this one has started, and such a pointer
+// may be read through the read-only path, or ahead of the wait.  Both calls do nothing in a launch that is not chained.
 // Frames that share the SMs with other streams' frames are not chained: a
 // waiting CTA holds room that the other frames' kernels use.
 // A lone 1080p chunk frame 310 -> 288 us, an LOD frame 305 -> 291, 256 x 256

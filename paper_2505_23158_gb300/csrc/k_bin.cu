@@ -199,13 +199,13 @@ __device__ __forceinline__ int64_t emit_first(uint32_t t, int rest, int& size) {
 // record's keys took 25.8.
 constexpr uint32_t kWarpKeys = 32;   // at most 2^10 (warp_records)
 __global__ void __launch_bounds__(kEmitThreads)
-emit_fused_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis,
-                  const uint2* __restrict__ rec_rect, int bin_log2, int32_t bins_x, int64_t n_keys,
-                  uint32_t* __restrict__ tile_key, uint32_t* __restrict__ tile_val, int rbits,
-                  int passes, uint32_t last_mask, uint32_t* __restrict__ digit_hist,
-                  uint32_t* __restrict__ status, uint32_t* __restrict__ counter,
-                  uint32_t* __restrict__ err, const unsigned long long* __restrict__ d_nvis,
-                  const unsigned long long* __restrict__ d_nkeys) {
+emit_fused_kernel(const uint32_t* sorted_rec, int64_t n_vis,
+                  const uint2* rec_rect, int bin_log2, int32_t bins_x, int64_t n_keys,
+                  uint32_t* tile_key, uint32_t* tile_val, int rbits,
+                  int passes, uint32_t last_mask, uint32_t* digit_hist,
+                  uint32_t* status, uint32_t* counter,
+                  uint32_t* err, const unsigned long long* d_nvis,
+                  const unsigned long long* d_nkeys) {
     chain_wait();
     // with device counts, n_vis and n_keys are capacities: the counts decide
     // which CTAs work and the keys must fit n_keys
@@ -296,7 +296,7 @@ emit_fused_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis,
 // the records' rects are read twice instead.
 constexpr int64_t kEmitSplitMin = 1ll << 21;                 // record capacity above which it is used
 
-__device__ __forceinline__ uint32_t rec_bin_rect(const uint2* __restrict__ rec_rect, uint32_t rec,
+__device__ __forceinline__ uint32_t rec_bin_rect(const uint2* rec_rect, uint32_t rec,
                                                  int bin_log2, uint32_t& x0, uint32_t& y0, uint32_t& w) {
     const uint2 p = rec_rect[rec];   // pixel range -> tile range -> bin range
     x0 = ((p.x & 0xffffu) / kTile) >> bin_log2;
@@ -314,9 +314,9 @@ __device__ __forceinline__ int64_t device_count(int64_t cap, const unsigned long
 
 template <int kEmitRecs>
 __global__ void __launch_bounds__(kEmitThreads)
-emit_count_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
-                  const unsigned long long* __restrict__ d_nvis, const uint2* __restrict__ rec_rect,
-                  int bin_log2, uint32_t* __restrict__ tile_sum, uint32_t* __restrict__ err) {
+emit_count_kernel(const uint32_t* sorted_rec, int64_t n_vis_cap,
+                  const unsigned long long* d_nvis, const uint2* rec_rect,
+                  int bin_log2, uint32_t* tile_sum, uint32_t* err) {
     constexpr int kEmitTileRecs = kEmitThreads * kEmitRecs;
     __shared__ uint32_t s_part[kEmitThreads / 32];
     chain_wait();
@@ -349,8 +349,8 @@ emit_count_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
 // One CTA of 1024 threads: the tile counts become exclusive offsets in place;
 // their total must equal the keys the projection counted and fit key_cap.
 __global__ void __launch_bounds__(1024)
-emit_scan_kernel(int tile_recs, uint32_t* __restrict__ tile_sum, int64_t n_vis_cap, const unsigned long long* __restrict__ d_nvis,
-                 int64_t key_cap, const unsigned long long* __restrict__ d_nkeys, uint32_t* __restrict__ err) {
+emit_scan_kernel(int tile_recs, uint32_t* tile_sum, int64_t n_vis_cap, const unsigned long long* d_nvis,
+                 int64_t key_cap, const unsigned long long* d_nkeys, uint32_t* err) {
     __shared__ uint32_t s_scan[33];
     chain_wait();
     const int64_t n_vis = device_count(n_vis_cap, d_nvis);
@@ -372,11 +372,11 @@ emit_scan_kernel(int tile_recs, uint32_t* __restrict__ tile_sum, int64_t n_vis_c
 
 template <int kEmitRecs>
 __global__ void __launch_bounds__(kEmitThreads)
-emit_write_kernel(const uint32_t* __restrict__ sorted_rec, int64_t n_vis_cap,
-                  const unsigned long long* __restrict__ d_nvis, const uint2* __restrict__ rec_rect,
-                  int bin_log2, int32_t bins_x, int64_t key_cap, const uint32_t* __restrict__ tile_off,
-                  uint32_t* __restrict__ tile_key, uint32_t* __restrict__ tile_val, int rbits, int passes,
-                  uint32_t last_mask, uint32_t* __restrict__ digit_hist, uint32_t* __restrict__ err) {
+emit_write_kernel(const uint32_t* sorted_rec, int64_t n_vis_cap,
+                  const unsigned long long* d_nvis, const uint2* rec_rect,
+                  int bin_log2, int32_t bins_x, int64_t key_cap, const uint32_t* tile_off,
+                  uint32_t* tile_key, uint32_t* tile_val, int rbits, int passes,
+                  uint32_t last_mask, uint32_t* digit_hist, uint32_t* err) {
     constexpr int kEmitTileRecs = kEmitThreads * kEmitRecs;
     __shared__ uint32_t s_scan[33];
     __shared__ uint32_t s_nbig;

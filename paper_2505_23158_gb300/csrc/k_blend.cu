@@ -72,7 +72,7 @@ __device__ __forceinline__ f32x2 keep2(bool lo, bool hi, f32x2 a, f32x2 b) {
 // One record against the thread's two pixels (Eq. 1).  Returns the weights
 // T alpha (0 where the pixel skips or has stopped); T becomes the
 // transmittance after the record (below kStop where it has stopped).
-__device__ __forceinline__ void blend_pair(const char* __restrict__ rec, float pxf, float py0, PixelPair& p,
+__device__ __forceinline__ void blend_pair(const char* rec, float pxf, float py0, PixelPair& p,
                                            f32x2& wgt) {
     constexpr int kNext = sizeof(float4) * kBlendBatch;
     const float4 a = *reinterpret_cast<const float4*>(rec);
@@ -108,12 +108,12 @@ __device__ __forceinline__ void blend_tile(const BlendFrame& f, int tile) {
     __shared__ uint32_t s_met[4][kBlendBatch / 32];        // per block: which records reach it
     __shared__ __align__(8) uint16_t s_hit[4][kBlendBatch];   // per warp: their offsets
     const int32_t width = f.width, height = f.height, tiles_x = f.tiles_x;
-    const uint32_t* __restrict__ tile_val = f.tile_val;
+    const uint32_t* tile_val = f.tile_val;
     const uint32_t vmask = f.vmask, n_keys = f.n_keys, n_rec = f.n_rec;
-    const float4* __restrict__ rec_a = f.rec_a;
-    const float4* __restrict__ rec_b = f.rec_b;
-    const float* __restrict__ rec_c = f.rec_c;
-    const uint2* __restrict__ rec_rect = f.rec_rect;
+    const float4* rec_a = f.rec_a;
+    const float4* rec_b = f.rec_b;
+    const float* rec_c = f.rec_c;
+    const uint2* rec_rect = f.rec_rect;
     const int tx = tile % tiles_x, ty = tile / tiles_x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // warp w covers the 8x8 block (w & 1, w >> 1) of the tile; a lane owns

@@ -98,8 +98,8 @@ struct KeySplat {
 // once the near cull has passed.
 template <bool kPre = false>
 __device__ __forceinline__ bool key_splat(const DevScene& sc, const DevCamera& cam, float mxw,
-                                          float myw, float mzw, const float4* __restrict__ sso,
-                                          const float4* __restrict__ sq, int64_t idx, uint32_t g,
+                                          float myw, float mzw, const float4* sso,
+                                          const float4* sq, int64_t idx, uint32_t g,
                                           float mult, KeySplat& k, float4 so_pre = float4{},
                                           float4 q_pre = float4{}) {
     const float* R = cam.R;
@@ -208,8 +208,8 @@ __device__ __forceinline__ bool key_splat(const DevScene& sc, const DevCamera& c
 // one takes 135 us alone.
 template <int kSrc>
 __global__ void __launch_bounds__(kProjThreads, kSrc == kStore ? 8 : 6)
-project_kernel(ProjParams P, uint32_t* __restrict__ status, uint32_t* __restrict__ tile_counter,
-               uint32_t* __restrict__ err) {
+project_kernel(ProjParams P, uint32_t* status, uint32_t* tile_counter,
+               uint32_t* err) {
     __shared__ uint32_t s_tile, s_prefix;
     __shared__ uint32_t s_cnt[kProjThreads / 32];
     __shared__ unsigned long long s_keys, s_bkeys;

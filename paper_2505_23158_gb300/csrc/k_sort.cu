@@ -62,11 +62,11 @@ __global__ void hist_scan_kernel(uint32_t* hist) {
 
 template <int kIPT, bool kWriteKeys, bool kValues>
 __global__ void __launch_bounds__(kSortThreads, 4)
-onesweep_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-              uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n, int shift,
-              uint32_t dmask, const uint32_t* __restrict__ offsets, uint32_t* __restrict__ status,
-              uint32_t* __restrict__ counter, uint32_t* __restrict__ err, uint2* __restrict__ ranges,
-              int range_shift, uint32_t range_tiles, const unsigned long long* __restrict__ d_count,
+onesweep_pass(const uint32_t* kin, const uint32_t* vin,
+              uint32_t* kout, uint32_t* vout, int64_t n, int shift,
+              uint32_t dmask, const uint32_t* offsets, uint32_t* status,
+              uint32_t* counter, uint32_t* err, uint2* ranges,
+              int range_shift, uint32_t range_tiles, const unsigned long long* d_count,
               bool raw_counts) {
     constexpr int kTileN = kSortThreads * kIPT;
     __shared__ uint32_t s_whist[kWarps][kRadix];
