@@ -309,20 +309,10 @@ __global__ void __launch_bounds__(kBlendThreads, 8) blend_loop_kernel(BlendFrame
     }
 }
 
-// One launch for the tiles of several frames (a serving step): CTA b
-// composites tile b - tile_base of the last frame whose tile_base <= b.
-__global__ void __launch_bounds__(kBlendThreads, 8) blend_batch_kernel(BlendBatch bb) {
-    const uint32_t b = blockIdx.x;
-    int lo = 0, hi = bb.n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (bb.f[mid].tile_base <= b) lo = mid; else hi = mid - 1;
-    }
-    blend_tile<false>(bb.f[lo], (int)(b - bb.f[lo].tile_base));
-}
-
-// The same as a persistent grid: each CTA takes the next (frame, tile) item
-// of the step from the counter until all `total` are done.
+// One persistent launch for the tiles of several frames (a serving step): each
+// CTA takes the next (frame, tile) item b of the step from the counter until
+// all `total` are done; it is tile b - tile_base of the last frame whose
+// tile_base <= b.
 __global__ void __launch_bounds__(kBlendThreads, 8) blend_batch_loop_kernel(BlendBatch bb, uint32_t total,
                                                                          uint32_t* __restrict__ tile_ctr) {
     __shared__ uint32_t s_t;
@@ -454,17 +444,13 @@ void launch_blend_batch(const BlendFrame* frames, int n, cudaStream_t s, uint32_
         ++bb.n;
     }
     if (bb.n == 0) return;
-    if (tile_ctr) {
-        // as many CTAs as fit on the device at once (the step's compositing
-        // runs after every frame's earlier stages)
-        int per_sm = 1;
-        const int nsm = device_sms();
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, blend_batch_loop_kernel, kBlendThreads, 0);
-        const unsigned grid = (unsigned)std::min<int64_t>((int64_t)base, (int64_t)nsm * std::max(per_sm, 1));
-        blend_batch_loop_kernel<<<grid, kBlendThreads, 0, s>>>(bb, base, tile_ctr);
-        return;
-    }
-    blend_batch_kernel<<<base, kBlendThreads, 0, s>>>(bb);
+    // as many CTAs as fit on the device at once (the step's compositing runs
+    // after every frame's earlier stages)
+    int per_sm = 1;
+    const int nsm = device_sms();
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, blend_batch_loop_kernel, kBlendThreads, 0);
+    const unsigned grid = (unsigned)std::min<int64_t>((int64_t)base, (int64_t)nsm * std::max(per_sm, 1));
+    blend_batch_loop_kernel<<<grid, kBlendThreads, 0, s>>>(bb, base, tile_ctr);
 }
 
 void launch_importance(const DevCamera& cam, const uint2* ranges, const uint32_t* tile_val,
