@@ -140,7 +140,13 @@ typedef struct {
 
 /* Create a context on CUDA device `device`.  hbm_budget_bytes caps the
  * device memory the context may hold (scenes + scratch); 0 = no cap.
- * *out receives the context; destroy it with lodge_destroy. */
+ * *out receives the context; destroy it with lodge_destroy.
+ * The contexts of a device without a cap take their scratch and saved frames
+ * from one memory pool, which keeps up to 2 GiB of freed memory mapped
+ * between calls.  Other allocators of the process cannot use that memory
+ * until the last of these contexts is destroyed; the library itself gives it
+ * back, with the scratch of streams no call uses, before an allocation of its
+ * own fails. */
 lodge_status lodge_create(int device, size_t hbm_budget_bytes, lodge_ctx** out);
 
 /* Free every device and host resource of the context.  NULL is a no-op. */
@@ -244,7 +250,8 @@ lodge_status lodge_set_bin_size(lodge_ctx* ctx, int32_t log2_tiles);
  * (scratch sized by capacities, counts read at the end of the call); a
  * frame whose keys outgrow that capacity is rendered again
  * (lodge_profile.redone), so images and counters are those of rendering
- * each camera alone. */
+ * each camera alone.  A call that finds no memory for the scratch of several
+ * streams goes on with one. */
 lodge_status lodge_render(lodge_ctx* ctx, int32_t scene_id, lodge_mode mode,
                           const lodge_camera* cams, int32_t n_cams, float* d_rgb, void* stream,
                           int32_t save_for_backward, int64_t* handle_out,
@@ -293,8 +300,10 @@ lodge_status lodge_render_lod(lodge_ctx* ctx, int32_t scene_id, const lodge_came
  * maximum over all their views.  chunk < 0: the mode's active set per camera;
  * chunk >= 0: chunk `chunk`'s own active set for every camera, with no
  * blending (resident scenes only; the views of a chunk's visibility
- * filtering).  Synchronous on stream.  Errors: LODGE_E_INVALID,
- * LODGE_E_NOT_RESIDENT. */
+ * filtering).  Views of a resident scene take turns on several streams, as in
+ * lodge_render.  Synchronous on stream.  Errors: LODGE_E_INVALID,
+ * LODGE_E_NOT_RESIDENT; LODGE_E_BUDGET or LODGE_E_OOM if one view's scratch
+ * does not fit. */
 lodge_status lodge_importance(lodge_ctx* ctx, int32_t scene_id, lodge_mode mode, int32_t chunk,
                               const lodge_camera* cams, int32_t n_cams, float* d_score,
                               void* stream);
@@ -337,9 +346,10 @@ lodge_status lodge_render_params(lodge_ctx* ctx, int64_t n, const float* d_means
  *   d_rgb: H x W x 3 (device).
  *   d_score (device, total Gaussians, optional): when given, the frame also
  *     raises the importance scores (as lodge_importance) and cannot be saved.
- *   save_for_backward: keep the frame for lodge_render_backward, which then
- *     gives gradients of level train_level only, into arrays of that level's
- *     size (the other levels are fixed, as in the build).
+ *   save_for_backward: keep the frame for lodge_render_backward or
+ *     lodge_render_gradients, which then give gradients of level train_level
+ *     only, into arrays of that level's size (the other levels are fixed, as
+ *     in the build).
  * Synchronous on stream.  Errors: LODGE_E_INVALID (sizes, thresholds,
  * pointers, train_level), LODGE_E_OOM, LODGE_E_CUDA. */
 lodge_status lodge_render_params_lod(lodge_ctx* ctx, int32_t num_levels, const int64_t* level_n,

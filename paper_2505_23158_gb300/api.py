@@ -456,7 +456,7 @@ def kmeans_centers(positions, init, max_iter: int = 100):
 class _RenderParams(torch.autograd.Function):
     """Differentiable render of raw Gaussian parameters through the library's
     forward (lodge_render_params) and hand-written adjoint
-    (lodge_render_backward)."""
+    (lodge_render_gradients)."""
 
     @staticmethod
     def forward(fctx, means, log_scales, quats, logits, sh, lodge, cam, sh_degree, filter_var):
@@ -480,7 +480,7 @@ class _RenderParams(torch.autograd.Function):
 
 class _RenderLevelLod(torch.autograd.Function):
     """LOD render of several levels in which only one level's parameters are
-    trained: forward lodge_render_params_lod, adjoint lodge_render_backward
+    trained: forward lodge_render_params_lod, adjoint lodge_render_gradients
     restricted to that level."""
 
     @staticmethod

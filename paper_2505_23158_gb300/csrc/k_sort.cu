@@ -1,9 +1,10 @@
 // K5: stable LSD radix sort of u32 keys, with or without u32 values,
 // "onesweep" style: the digit histograms are known before the first pass (one
 // upfront histogram pass, or supplied by the caller), then each 8-bit digit
-// is scattered in a single pass in which a tile of pairs (3840, or 1024 for
-// inputs up to 2^20 so that small sorts still fill the SMs) learns its global
-// offsets by decoupled look-back over its predecessors' per-digit counts.
+// is scattered in a single pass in which a tile of pairs (3840; for inputs up
+// to 2^20 1024, so that small sorts still fill the SMs, or 2048 where other
+// frames share them) learns its global offsets by decoupled look-back over its
+// predecessors' per-digit counts.
 //
 // Used twice per frame: by FP32 depth (4 digits) over the visible records,
 // then by tile id over the emitted (tile, record) pairs, which yields the

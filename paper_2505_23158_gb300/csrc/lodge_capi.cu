@@ -2147,10 +2147,11 @@ lodge_status lodge_render_params(lodge_ctx* ctx, int64_t n, const float* d_means
 
 // LOD rendering of levels given as raw device parameters (supplementary
 // "LOD structure optimization steps": the build of level l fine-tunes G_l
-// with LOD rendering of the levels up to l, d_l drawn per step).  The levels
-// are activated into one gid-ordered store (finest first), Eq. 2 selects
-// each level's band at the camera centre with this frame's thresholds, and
-// the frame is rendered as any LOD frame.  With d_score it raises the
+// with LOD rendering of the levels up to l, d_l drawn per step).  Eq. 2
+// selects each level's band at the camera centre with this frame's thresholds
+// (from planes of the means, gid order, finest level first); everything else
+// is read from the caller's arrays in place and the frame is rendered as any
+// LOD frame.  With d_score it raises the
 // importance scores instead (K12); with save_for_backward the adjoint will
 // give gradients of level train_level only.
 lodge_status lodge_render_params_lod(lodge_ctx* ctx, int32_t num_levels, const int64_t* level_n,
