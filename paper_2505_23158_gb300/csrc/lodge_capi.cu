@@ -228,9 +228,13 @@ void release(lodge_ctx* ctx, DBuf& b, cudaStream_t s) {
     b.cap = 0;
 }
 
-// stage profiling: events around each stage, read after the next sync
+// stage profiling: events around each stage, read after the next sync (made
+// when a stage is first profiled)
 static void prof_begin(Slot& sl, int stage, cudaStream_t s) {
-    if (sl.prof_on && !sl.ev_pending[stage]) cudaEventRecord(sl.ev_beg[stage], s);
+    if (!sl.prof_on || sl.ev_pending[stage]) return;
+    if (!sl.ev_beg[stage]) cudaEventCreate(&sl.ev_beg[stage]);
+    if (!sl.ev_end[stage]) cudaEventCreate(&sl.ev_end[stage]);
+    cudaEventRecord(sl.ev_beg[stage], s);
 }
 static void prof_end(Slot& sl, int stage, cudaStream_t s, int launches) {
     sl.prof.launches[stage] += launches;
@@ -278,11 +282,6 @@ lodge_status create_slot(lodge_ctx* ctx, Slot** out) {
     CUDA_TRY(cudaMallocHost((void**)&sl->h_small, sizeof(uint32_t) * kSmWords * (2 + Slot::kRing)));
     sl->h_tail = sl->h_small + kSmWords;
     sl->h_ring = sl->h_tail + kSmWords;
-    for (int k = 0; k < Slot::kRing; ++k) CUDA_TRY(cudaEventCreateWithFlags(&sl->ring_ev[k], cudaEventDisableTiming));
-    for (int k = 0; k < LODGE_NUM_STAGES; ++k) {
-        CUDA_TRY(cudaEventCreate(&sl->ev_beg[k]));
-        CUDA_TRY(cudaEventCreate(&sl->ev_end[k]));
-    }
     std::lock_guard<std::recursive_mutex> lk(ctx->mu);
     *out = sl.get();
     ctx->slots.emplace_back(std::move(sl));
@@ -907,6 +906,7 @@ static lodge_status render_frame(lodge_ctx* ctx, Slot& sl, const DevScene& dsc, 
         sl.ring_next = (sl.ring_next + 1) % Slot::kRing;
         CUDA_TRY(cudaMemcpyAsync(sl.h_ring + (size_t)ring * kSmWords, sl.d_small, sizeof(uint32_t) * kSmWords,
                                  cudaMemcpyDeviceToHost, s));
+        if (!sl.ring_ev[ring]) CUDA_TRY(cudaEventCreateWithFlags(&sl.ring_ev[ring], cudaEventDisableTiming));
         CUDA_TRY(cudaEventRecord(sl.ring_ev[ring], s));
         pend->ring = ring;
         pend->used = true;
