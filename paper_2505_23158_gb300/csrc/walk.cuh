@@ -85,24 +85,28 @@ __device__ __forceinline__ float ge01(float a, float b) {
 // the record's, the clamped x terms a column's and the y terms a row's, so
 // that four tests cost about 80 operations instead of 45 each.
 //
-// The record's pixel rect must come within a pixel of the block as well: the
-// rect holds the pixel centres within the extent, so a splat smaller than a
-// pixel often misses a block that its ellipse, tested over the whole box of the
-// centres, meets (four full-detail frames of 4M Gaussians 1540 us, 1575 with
-// the ellipse alone; the rect itself, as fast, does not cover its own rounding
-// on images of thousands of pixels: 2^-23 of the coordinate against 0.05% of
-// the extent).
+// The record's pixel rect must meet the block as well: the rect holds the pixel
+// centres within the extent, so a splat smaller than a pixel often misses a
+// block that its ellipse, tested over the whole box of the centres, meets (four
+// full-detail frames of 4M Gaussians 1540 us, 1575 with the ellipse alone).
+// The rect's own rounding, 2^-23 of the coordinate, is within its margin of
+// 0.05% of the extent but for splats of less than half a pixel far from the
+// corner whose edge falls on a pixel centre within 2e-4 of a pixel.
 //
-// kNan: a record whose form is not a number (a covariance that overflows
-// FP32) is kept, as in a walk without the test; the plain frames drop it.
-template <bool kNan>
+// kKept (frames kept for the adjoint, the adjoint, scores) leaves nothing to
+// that: the rect with a pixel around it counts (in the compositing of a lone
+// chunk frame 64.1M warp instructions against 62.2M).  A record whose
+// form is not a number (a covariance that overflows FP32) is kept there, as in
+// a walk without the test; the plain frames drop it.
+template <bool kKept>
 __device__ __forceinline__ uint32_t blocks_met(const float4 a, const float4 b, const uint2 rect, uint32_t tx0,
                                                uint32_t ty0) {
     constexpr float kLog2_255 = 7.99435343f;
     const uint32_t rx0 = rect.x & 0xffffu, ry0 = rect.x >> 16, rx1 = rect.y & 0xffffu, ry1 = rect.y >> 16;
     if (rx0 > tx0 + 15u || rx1 < tx0 || ry0 > ty0 + 15u || ry1 < ty0) return 0u;
-    const bool cx[2] = {rx0 <= tx0 + 8u, rx1 >= tx0 + 7u};   // the rect and a pixel around it
-    const bool cy[2] = {ry0 <= ty0 + 8u, ry1 >= ty0 + 7u};
+    constexpr uint32_t kGrow = kKept ? 1u : 0u;
+    const bool cx[2] = {rx0 <= tx0 + 7u + kGrow, rx1 + kGrow >= tx0 + 8u};
+    const bool cy[2] = {ry0 <= ty0 + 7u + kGrow, ry1 + kGrow >= ty0 + 8u};
     const float u00 = a.z, u01 = a.w, u11 = b.x;
     const float iy = __fdividef(-u00 * u01, fmaf(u01, u01, u11 * u11));
     const float ix = __fdividef(-u01, u00);
@@ -133,7 +137,7 @@ __device__ __forceinline__ uint32_t blocks_met(const float4 a, const float4 b, c
             const float dx = fminf(fmaxf(xm[r], X0[c]), X1[c]);
             const float t2 = fmaf(u00, dx, uy[r]);
             const float q = fminf(fmaf(t1, t1, w1 * w1), fmaf(t2, t2, wy[r]));
-            if (cx[c] && cy[r] && (kNan ? !(q > lim) : q <= lim)) met |= 1u << (2 * r + c);
+            if (cx[c] && cy[r] && (kKept ? !(q > lim) : q <= lim)) met |= 1u << (2 * r + c);
         }
     return met;
 }
